@@ -415,8 +415,13 @@ int tail_start(const mg_ctx *c)
 // zero: p is taken as zero on entry (a cycle from a zero guess): the coarsest solve overwrites it,
 // the coarse tail zeroes it in its kernel, and the per-colour passes start with a pass that reads
 // no iterate, so no separate clearing pass is needed (the fused sweeps and nu1 = 0 clear it first)
+// again: the last thing done to p was a cycle with this b.  Its last pass was the red one of a
+// post-smoothing sweep, so this cycle's first red pass would compute the red values that stand there
+// from the same black ones: it is left out (the same iterate bit for bit, one of the finest level's
+// 2 (nu1 + nu2) passes less)
 template <typename T>
-int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T *p, bool zero = false)
+int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T *p, bool zero = false,
+           bool again = false)
 {
     cudaStream_t s = c->s;
     const Dims d = c->dims[l];
@@ -464,6 +469,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     // the first pass reads no iterate when p starts at zero; otherwise clear p first
     bool zpass = zero && !fused && c->o.nu1 >= 1;
     if (zero && !zpass) CK(cudaMemsetAsync(p, 0, d.n() * sizeof(T), s));
+    bool skip = again && !fused && c->o.nu1 >= 1 && c->o.nu2 >= 1;  // the first red pass
     // one red-black sweep, `first` colour first
     auto sweep = [&](int first) -> int {
         ProfScope ps(c, MG_PROF_SMOOTH, fine);
@@ -476,16 +482,18 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
         } else if (sp.half) {
             if constexpr (std::is_same<T, float>::value) {
                 const int r0 = alternate ? (npass + 1) & 1 : 0;
-                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first, s, urow, arow, r0, zpass, &c->sf0));
-                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first ^ 1, s, urow, arow, r0 ^ (alternate ? 1 : 0),
-                                           false, &c->sf0));
-                npass += 2;
+                if (!skip)
+                    CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first, s, urow, arow, r0, zpass, &c->sf0));
+                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first ^ 1, s, urow, arow,
+                                           skip ? r0 : r0 ^ (alternate ? 1 : 0), false, &c->sf0));
+                npass += skip ? 1 : 2;
             }
         } else {
-            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first, s, 0, -1, zpass));
+            if (!skip) CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first, s, 0, -1, zpass));
             CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first ^ 1, s));
         }
         zpass = false;
+        skip = false;
         return MG_OK;
     };
     for (int it = 0; it < c->o.nu1; it++) CKS(sweep(0));
@@ -494,7 +502,9 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
         ProfScope ps(c, MG_PROF_RESTRICT, fine);
         // descending after an ascending last pass (an even number of passes, the last ascending)
         const int rrev = alternate && npass > 0 && (npass & 1) == 0 ? 1 : 0;
-        CK(mg::launch_resid_restrict<T>(d, ih2, L[l], b, cur, C.b, s, sp, urow, rrev));
+        const LevelArrays<T> *S = nullptr;
+        if constexpr (std::is_same<T, float>::value) S = l == 0 ? &c->sf0 : nullptr;
+        CK(mg::launch_restrict<T>(d, ih2, L[l], b, cur, C.b, s, sp, urow, arow, rrev, S));
     }
     npass = 0;
     {
@@ -506,7 +516,10 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     }
     {
         ProfScope ps(c, MG_PROF_PROLONG, fine);
-        CK(mg::launch_prolong<T>(d, C.p, L[l].dinv, cur, s, sp, urow));
+        if (c->o.nu2 >= 1)  // a black pass follows: the red cells alone
+            CK(mg::launch_prolong_red<T>(d, C.p, L[l].dinv, cur, s, sp, urow, arow));
+        else
+            CK(mg::launch_prolong<T>(d, C.p, L[l].dinv, cur, s, sp, urow));
     }
     for (int it = 0; it < c->o.nu2; it++) CKS(sweep(1));
     if (cur != p) CK(cudaMemcpyAsync(p, cur, d.n() * sizeof(T), cudaMemcpyDeviceToDevice, s));
@@ -706,14 +719,14 @@ int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st
         cyc++;
         if (mixed) {
             for (int ic = 0; ic < c->o.inner_cycles; ic++)
-                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, c->L32[0].p, ic == 0));
+                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, c->L32[0].p, ic == 0, ic > 0));
             CK(mg::launch_accumulate(d, c->L64[0].dinv, c->L32[0].p, p, c->dscal, scale_slot, s, c->split0));
             std::swap(scale_slot, next_slot);
             ProfScope ps(c, MG_PROF_RESID64, true);
             CK(mg::launch_resid_cast(d, ih2, c->L64[0], c->b0, p, c->L32[0].b, c->partials, c->dscal, scale_slot,
                                      next_slot, s, c->split0));
         } else {
-            CKS(vcycle<double>(c, c->L64, 0, c->b0, p));
+            CKS(vcycle<double>(c, c->L64, 0, c->b0, p, false, cyc > 1));
             if (cyc % c->o.check_every != 0 && cyc < c->o.max_cycles) continue;
             ProfScope ps(c, MG_PROF_RESID64, true);
             CK(mg::launch_resid_norm(d, ih2, c->L64[0], c->b0, p, c->partials, c->dscal, s));
@@ -865,9 +878,9 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
         if (c->o.precond == 1) {
             CK(mg::launch_jacobi(n, -c->hs[0] * c->hs[0], c->L64[0].dinv, c->kr, z, s));
         } else if (mixed) {
-            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0));
+            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0, v > 0));
         } else {
-            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0));
+            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0, v > 0));
         }
         return MG_OK;
     };

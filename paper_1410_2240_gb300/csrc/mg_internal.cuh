@@ -150,11 +150,17 @@ cudaError_t launch_rb_sweep_tma(Dims d, float h2, const LevelArrays<float> &L, c
 template <typename T>
 cudaError_t launch_rb_sweep(Dims d, T h2, const LevelArrays<T> &L, const T *b, const T *p_old, T *p_new, int first,
                             cudaStream_t s);
-// b and p of the fine level in the layout sp (FP32 only may be split); bc natural; rev (FP32): blocks
-// take the coarse planes in descending order
+// b and p of the fine level in the layout sp (FP32 only may be split), bc natural; on a colour-split
+// level with nx % 8 == 0: urow / arow (arow replaces urow where the sweeps use it) and S as for
+// launch_smooth_split, required, and rev: blocks take the coarse planes in descending order
 template <typename T>
-cudaError_t launch_resid_restrict(Dims fine, T ih2, const LevelArrays<T> &L, const T *b, const T *p, T *bc,
-                                  cudaStream_t s, Split sp = {}, const float *urow = nullptr, int rev = 0);
+cudaError_t launch_restrict(Dims fine, T ih2, const LevelArrays<T> &L, const T *b, const T *p, T *bc, cudaStream_t s,
+                            Split sp = {}, const float *urow = nullptr, const float4 *arow = nullptr, int rev = 0,
+                            const LevelArrays<T> *S = nullptr);
+// prolongation before a black colour pass: corrects the red cells alone
+template <typename T>
+cudaError_t launch_prolong_red(Dims fine, const T *ec, const T *dinv, T *p, cudaStream_t s, Split sp = {},
+                               const float *urow = nullptr, const float4 *arow = nullptr);
 template <typename T>
 // urow (optional, FP32): the fine level's uniform-row values (cells of uniform rows are all live)
 cudaError_t launch_prolong(Dims fine, const T *ec, const T *dinv, T *p, cudaStream_t s, Split sp = {},

@@ -1,0 +1,70 @@
+"""The passes of a V-cycle that depend on its smoothing counts: the prolongation corrects the red
+cells alone where a black pass follows (nu2 >= 1), all cells otherwise; a cycle that continues
+the one before it leaves its first red pass out (nu1, nu2 >= 1).
+
+Bounds: a V-cycle against the oracle's with the same counts to 1e-12 (FP64) and 3e-6 of max|p|
+(FP32), the bounds of the other cycle tests.  Cycles run by a solve against the same number of
+single cycles: the kernels and their order are the same, so the iterates agree up to the mean
+that the solve removes at its end (one subtraction, taken here in another order of summation):
+1e-13 of max|p|.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1410_2240_gb300 import synth
+
+from _gpu_util import case_rhs, dev, host, rel
+
+pytestmark = pytest.mark.gpu
+
+# cells along x: a multiple of 8, of 4 alone and of 2 alone; two to four levels; small coarsest grids
+# (their oracle inverse is a dense eigen-decomposition)
+SHAPES = [(48, 16, 24), (36, 16, 16), (20, 16, 24), (10, 8, 8), (16, 8, 8)]
+
+
+@pytest.fixture(scope="module")
+def mgp():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1410_2240_gb300 import mgproj
+    return mgproj
+
+
+def _setup(mgp, shape, **kw):
+    case = synth.small_case(*shape, solid="ellipsoid", seed=51)
+    beta_o = O.face_coeffs(case.phi, case.solid, case.lam)
+    b = O.remove_mean(case_rhs(case, beta_o), *O.components(beta_o))
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    return case, beta_o, b, mgp.Context(beta, case.h, coarse_max_cells=2048, **kw)
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (1, 1), (0, 2), (2, 0)])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_cycle_with_smoothing_counts_matches_oracle(mgp, shape, nu):
+    for prec in ("fp64", "mixed"):
+        case, beta_o, b, ctx = _setup(mgp, shape, prec=prec, nu1=nu[0], nu2=nu[1])
+        mg = O.MG(beta_o, case.h, nu1=nu[0], nu2=nu[1])
+        p = np.zeros(b.shape)
+        for it in range(2):
+            pd = dev(p)
+            p = mg.vcycle(b, p)
+            ctx.vcycle(dev(b), pd)
+            if prec == "fp64":
+                assert rel(host(pd), p) <= 1e-12, it
+            else:
+                assert np.abs(host(pd) - p).max() <= 3e-6 * np.abs(p).max(), it
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_continued_cycles_are_the_single_ones(mgp, shape):
+    case, beta_o, b, ctx = _setup(mgp, shape, max_cycles=3)
+    p, st = ctx.solve(dev(b), tol=1e-30, allow_not_converged=True)
+    q = dev(np.zeros(b.shape))
+    for _ in range(3):
+        ctx.vcycle(dev(b), q)
+    lab, nc = O.components(beta_o)
+    q = O.remove_mean(host(q), lab, nc)
+    assert st.cycles == 3
+    assert np.abs(host(p) - q).max() <= 1e-13 * np.abs(q).max()
