@@ -104,10 +104,10 @@ typedef struct {
     int coarse_graph;     /* 1: replay the coarse-grid part of each V-cycle (all levels below the
                              finest) as one CUDA graph captured on first use on a private stream;
                              0: launch its kernels one by one.  Identical results [1] */
-    int coarse_tail;      /* 1: the smallest levels below the finest (each field of at most a few
-                             thousand cells) are smoothed, restricted and prolonged by one CTA in
-                             two launches around the coarsest solve instead of a launch per pass;
-                             0: a launch per pass.  Identical results [1] */
+    int coarse_tail;      /* 1: the levels of at most 8192 cells below the finest, the coarsest solve
+                             included (up to 1024 cells), run in one launch of one thread-block
+                             cluster instead of a launch per pass; 0: a launch per pass.  Identical
+                             results [1] */
     int precond;          /* preconditioner of the conjugate gradients (krylov = 1): 0 inner_cycles
                              multigrid V-cycles; 1 Jacobi (the inverse diagonal, z = D^-1 r; MG_FP64
                              only), the diagonally preconditioned CG the Poisson-solver section

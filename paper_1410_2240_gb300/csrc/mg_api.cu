@@ -58,6 +58,14 @@ namespace mg {
 void set_last_error(const char *msg) { g_err = msg; }
 }  // namespace mg
 
+// The coarse tail of a context in one precision: its first level (-1: none) and the kernel's
+// arguments but for that level's b and p
+template <typename T>
+struct TailPlan {
+    int first = -1;
+    mg::TailArgs<T> a{};
+};
+
 struct mg_ctx {
     mg_grid g{};
     mg_opts o{};
@@ -67,6 +75,8 @@ struct mg_ctx {
     std::vector<double> hs;
     std::vector<LevelArrays<double>> L64;
     std::vector<LevelArrays<float>> L32;
+    TailPlan<double> tail64;
+    TailPlan<float> tail32;
     std::vector<double *> palt64;  // second iterate buffer per level for fused sweeps (null if unused)
     std::vector<float *> palt32;
     // conjugate-gradient vectors (krylov = 1): FP64 r, d, q; z, z_old (FP64 cycles) or a
@@ -368,6 +378,13 @@ double *palt_of<double>(mg_ctx *c, int l) { return c->palt64.empty() ? nullptr :
 template <>
 float *palt_of<float>(mg_ctx *c, int l) { return c->palt32.empty() ? nullptr : c->palt32[l]; }
 
+template <typename T>
+const TailPlan<T> &tail_of(const mg_ctx *c);
+template <>
+const TailPlan<double> &tail_of<double>(const mg_ctx *c) { return c->tail64; }
+template <>
+const TailPlan<float> &tail_of<float>(const mg_ctx *c) { return c->tail32; }
+
 // fused sweeps pay off on levels with at least one full 32 x 8 tile and 8 planes
 bool fused_level(const Dims &d) { return d.nx >= 32 && d.ny >= 8 && d.nz >= 8; }
 
@@ -400,16 +417,56 @@ inline cudaError_t launch_sweep_tma(Dims, double, const LevelArrays<double> &, c
 template <typename T>
 int coarse_correction_graph(mg_ctx *c, const std::vector<LevelArrays<T>> &L);
 
-// First level of the coarse tail in precision T: the largest level below the finest, above the
-// coarsest, whose six fields (p, b, three face arrays, dinv) fit in an SM's L1; -1 if none.
-constexpr size_t kTailBytes = 200 * 1024;
+// The coarse tail in precision T: its first level (the largest below the finest and above the coarsest
+// whose slabs, with those of all levels below, fit in the shared memory of a cluster's CTAs; -1 if
+// none, or if the coarsest grid is larger than a cluster should solve) and its layout.
 template <typename T>
-int tail_start(const mg_ctx *c)
+int tail_layout(const mg_ctx *c, const std::vector<LevelArrays<T>> &L, int ctas, mg::TailArgs<T> &a)
 {
-    if (!c->o.coarse_tail) return -1;
-    for (int l = 1; l + 1 < c->nlev; l++)
-        if (c->dims[l].n() * 6 * sizeof(T) <= kTailBytes && c->nlev - l <= mg::kTailMaxLevels) return l;
+    if (c->ncoarse > mg::kTailCoarse) return -1;
+    for (int l = 1; l + 1 < c->nlev; l++) {
+        if (c->nlev - l > mg::kTailMaxLevels || c->dims[l].n() > mg::kTailCellsMax) continue;
+        a.nlev = c->nlev - l;
+        a.ctas = ctas;
+        size_t n = 0;  // elements per CTA
+        bool fits = true;
+        for (int q = 0; q < a.nlev; q++) {
+            const Dims d = c->dims[l + q];
+            mg::TailLevel<T> &v = a.lev[q];
+            v.nx = d.nx;
+            v.ny = d.ny;
+            v.nz = d.nz;
+            v.P = (d.nz + ctas - 1) / ctas;
+            v.h2 = (T)(c->hs[l + q] * c->hs[l + q]);
+            v.ih2 = (T)(1.0 / (c->hs[l + q] * c->hs[l + q]));
+            v.L = L[l + q];
+            v.fnx = mg::make_fastdiv((unsigned)d.nx);
+            v.fhx = mg::make_fastdiv((unsigned)std::max(d.nx / 2, 1));
+            v.fny = mg::make_fastdiv((unsigned)d.ny);
+            v.fP = mg::make_fastdiv((unsigned)v.P);
+            const size_t plane = (size_t)d.nx * d.ny, slab = plane * v.P;
+            const bool smoothed = q + 1 < a.nlev;
+            fits = fits && (!smoothed || slab <= 2 * (size_t)mg::kTailCells * mg::kTailThreads);
+            unsigned *const off[6] = {&v.op, &v.ob, &v.ox, &v.oy, &v.oz, &v.od};
+            for (int f = 0; f < (smoothed ? 6 : 2); f++) {
+                const size_t pad = smoothed && f == 0 ? d.nx / 2 : 0;  // the row of zeros before p
+                *off[f] = (unsigned)std::min<size_t>(n + pad, 0xffffffffu);
+                n += slab + pad + (smoothed ? d.nx : 0) + (f == 4 ? plane : 0);  // and after each colour
+            }
+        }
+        n = (n * sizeof(T) + 15) / 16 * 16;
+        a.sb_bytes = (unsigned)std::min<size_t>(n, 0xffffffffu);
+        a.smem = n + (size_t)c->ncoarse * sizeof(double);
+        if (fits && a.smem <= mg::kTailSmem) return l;
+    }
     return -1;
+}
+
+template <typename T>
+int tail_start(const mg_ctx *c, const std::vector<LevelArrays<T>> &L, mg::TailArgs<T> &a)
+{
+    const int ctas = c->o.coarse_tail ? mg::tail_ctas<T>() : 0;
+    return ctas > 0 ? tail_layout<T>(c, L, ctas, a) : -1;
 }
 
 // zero: p is taken as zero on entry (a cycle from a zero guess): the coarsest solve overwrites it,
@@ -429,27 +486,12 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
         CK(mg::launch_coarse_solve<T>(c->ncoarse, c->M, b, p, s));
         return MG_OK;
     }
-    if (l == tail_start<T>(c)) {  // this level and all below: one CTA, two launches
-        mg::TailArgs<T> a{};
-        a.nlev = c->nlev - l;
-        a.nu1 = c->o.nu1;
-        a.nu2 = c->o.nu2;
-        a.zero0 = zero ? 1 : 0;
-        for (int q = 0; q < a.nlev; q++) {
-            const int lv = l + q;
-            const Dims dl = c->dims[lv];
-            a.lev[q] = mg::TailLevel<T>{dl.nx, dl.ny, dl.nz, (T)(c->hs[lv] * c->hs[lv]),
-                                        (T)(1.0 / (c->hs[lv] * c->hs[lv])), L[lv],
-                                        mg::make_fastdiv((unsigned)(dl.nx + 1) / 2), mg::make_fastdiv((unsigned)dl.ny),
-                                        mg::make_fastdiv((unsigned)std::max(dl.nx / 2, 1)),
-                                        mg::make_fastdiv((unsigned)std::max(dl.ny / 2, 1))};
-        }
+    const TailPlan<T> &tail = tail_of<T>(c);
+    if (l == tail.first && zero) {  // this level and all below: one cluster, one launch
+        mg::TailArgs<T> a = tail.a;
         a.lev[0].L.b = const_cast<T *>(b);
         a.lev[0].L.p = p;
-        const LevelArrays<T> &Lc = L[c->nlev - 1];
-        CK(mg::launch_tail_down<T>(a, s));
-        CK(mg::launch_coarse_solve<T>(c->ncoarse, c->M, Lc.b, Lc.p, s));
-        CK(mg::launch_tail_up<T>(a, s));
+        CK(mg::launch_tail<T>(a, s));
         return MG_OK;
     }
     const T h2 = (T)(c->hs[l] * c->hs[l]);
@@ -1152,6 +1194,14 @@ int mg_setup(mg_ctx **out, const mg_grid *g, const double *const face_coeffs[3],
                 return bail(fail(MG_ERR_CUDA, "mg_setup: event creation failed"));
             }
     }
+    auto plan = [&](auto &t, const auto &L) {
+        t.first = tail_start(c, L, t.a);
+        t.a.nu1 = o.nu1;
+        t.a.nu2 = o.nu2;
+        t.a.M = c->M;
+    };
+    if (c->o.prec == MG_MIXED) plan(c->tail32, c->L32);
+    else plan(c->tail64, c->L64);
     st = compute_hierarchy(c, face_coeffs);
     if (st != MG_OK) return bail(st);
     c->ms_setup = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();

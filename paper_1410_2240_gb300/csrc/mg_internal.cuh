@@ -89,20 +89,34 @@ struct Split {
     FastDiv fnx, fny;  // division by nx and ny (the row and plane of a natural index)
 };
 
-// The coarse tail: levels lev[0] (the largest) .. lev[nlev-1] (the coarsest) of the hierarchy,
-// run by one CTA.  Each level's b and p are the ones a V-cycle on it would receive.
+// The coarse tail: levels lev[0] (the largest) .. lev[nlev-1] (the coarsest) of the hierarchy, kept in
+// the shared memory of a cluster of `ctas` CTAs (k_tail).  lev[0].L.b is the right-hand side and lev[0].L.p
+// receives the correction of a cycle from zero; the other levels' b and p stay inside.
 constexpr int kTailMaxLevels = 8;
+constexpr int kTailThreads = 256, kTailCells = 2;  // per CTA, and cells of a colour per thread at most
+// Cells of the tail's first level at most.  A pass in the cluster takes two trips between its SMs, about
+// 0.7 us, as long as its cells are few per SM; a launch in the coarse-grid graph 1.5 us.  First level of
+// 4096 cells against a launch per pass for it (coarse-grid correction, us): FP32 35 against 41, FP64
+// 48 against 54; of 13824 cells: FP32 48 and 49, FP64 76 and 72; of 32768: 37 and 35, 62 and 48 (the
+// FP64 unit of 16 SMs).
+constexpr size_t kTailCellsMax = 8192;
+constexpr size_t kTailSmem = 128 * 1024;   // shared memory per CTA at most (8192 FP64 cells need half)
+constexpr int kTailCoarse = 1024;          // cells of the coarsest grid at most
 template <typename T>
 struct TailLevel {
     int nx, ny, nz;
+    int P;                               // planes per CTA
+    unsigned op, ob, ox, oy, oz, od;     // offsets in a CTA's memory (elements): p, b, faces, inverse diagonal
     T h2, ih2;
     LevelArrays<T> L;
-    FastDiv fhx, fny, fcx, fcy;  // division by (nx + 1) / 2, ny, nx / 2 and ny / 2
+    FastDiv fnx, fhx, fny, fP;           // division by nx, nx / 2, ny, P
 };
 template <typename T>
 struct TailArgs {
-    int nlev, nu1, nu2;
-    int zero0;  // nonzero: lev[0].p starts at zero (zeroed here, not by the caller)
+    int nlev, nu1, nu2, ctas;
+    unsigned sb_bytes;                   // offset of the coarsest right-hand side in FP64
+    size_t smem;                         // bytes per CTA
+    const double *M;                     // the coarsest grid's inverse
     TailLevel<T> lev[kTailMaxLevels];
 };
 
@@ -167,12 +181,11 @@ cudaError_t launch_prolong(Dims fine, const T *ec, const T *dinv, T *p, cudaStre
                            const float *urow = nullptr);
 template <typename T>
 cudaError_t launch_coarse_solve(int n, const double *M, const T *b, T *e, cudaStream_t s);
-// the coarse tail's descent (pre-smoothing, restriction down to lev[nlev-1].b) and ascent
-// (prolongation of lev[nlev-1].p, post-smoothing up to lev[0].p); the coarsest solve runs between
+// a cluster's CTAs on the current device (0: none); the tail's launch
 template <typename T>
-cudaError_t launch_tail_down(const TailArgs<T> &a, cudaStream_t s);
+int tail_ctas();
 template <typename T>
-cudaError_t launch_tail_up(const TailArgs<T> &a, cudaStream_t s);
+cudaError_t launch_tail(const TailArgs<T> &a, cudaStream_t s);
 
 // connected components of the live cells (joined by open faces): label[c] = the smallest cell
 // index of c's component (-1 on dead cells); ctr[0] = number of components, ctr[1] != 0 if a

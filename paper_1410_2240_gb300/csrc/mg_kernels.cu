@@ -5,9 +5,11 @@
 // bx[.][.][0] is the wall (0).  The high wall face is not stored (closed).
 // A "live" cell has at least one open face (dinv > 0); other cells (solid or
 // isolated) hold p = 0 and are excluded from means and norms.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <type_traits>
@@ -206,7 +208,6 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // clear sign bit; the coefficients, inverse diagonals and live masks it is applied to are never
 // NaN for finite input.  zero_bits(x) equals x == 0 for every x.
 __device__ __forceinline__ bool pos_bits(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool pos_bits(float x) { return __float_as_int(x) > 0; }
 __device__ __forceinline__ bool zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ bool zero_bits(float x) { return (__float_as_int(x) << 1) == 0; }
 
@@ -890,7 +891,7 @@ __device__ __forceinline__ void restrict_box(int I, int J, int K, int nx, int ny
             P2 none;  // an absent outer neighbour: a closed face
             none.x = none.y = T(0);
             pc[dk][dj] = pair_q(p, c, q);
-            xl[dk][dj] = L.bx[c];
+            xl[dk][dj] = xlo ? L.bx[c] : T(0);
             xh[dk][dj] = xhi ? L.bx[c + 2] : T(0);
             pxl[dk][dj] = xlo ? val_q(p, c - 1, q) : T(0);
             pxh[dk][dj] = xhi ? val_q(p, c + 2, q) : T(0);
@@ -1008,7 +1009,7 @@ __global__ void k_restrict4(int nx, int ny, int nz, float ih2, LevelArrays<float
             } else {
                 const size_t e = q ? half : 0, o = q ? 0 : half;  // even and odd cells of the row
                 const float2 xf = ld2(S.bx + e, m);
-                x0 = xf.x;
+                x0 = xlo ? xf.x : 0.f;
                 x1 = xf.y;
                 x2 = xhi ? S.bx[e + m + 2] : 0.f;
                 if (dj) {  // the low faces of the row above
@@ -1423,101 +1424,251 @@ __global__ void k_coarse_solve(int n, const double *__restrict__ M, const T *__r
 }
 
 // ---------------------------------------------------------------------------
-// Coarse tail.  On the smallest levels (a few thousand cells) every colour pass, restriction and
-// prolongation is a launch far longer than its work.  One CTA runs them in sequence instead,
-// phases separated by __syncthreads (a level's fields stay in the SM's L1 between phases).  The
-// per-cell arithmetic is the per-pass kernels' own (smooth_cell, restrict_cell, prolong_corr) and
-// every cell of a pass is independent of the others, so the results are identical.  The fields
-// are written and read within the kernel, so they are read through plain pointers (never the
-// read-only path).
+// Coarse tail: one thread-block cluster runs all of a V-cycle from a level of some 10^4 cells down, the
+// exact solve on the coarsest grid included, in one launch.  A pass over such a level is far shorter
+// than a launch: as a graph of launches each of its ~10 passes took 1.5 us, and in one CTA, as the
+// tail ran before, a level of 16^3 cells was bound by that SM's instruction issue (FP32) or FP64 unit.
+// Here the levels live in the shared memory of the cluster's CTAs:
+//   * a level's planes are dealt out in slabs of P = ceil(nz / CTAs), stored colour by colour, so
+//     that a pass reads consecutive words;
+//   * a thread keeps the coefficients of its cells (at most kTailCells of each colour) in registers
+//     for all sweeps of a level, and a pass is six loads of the other colour, the update and a store;
+//   * the planes beside the slab are read from the neighbour CTA's shared memory (distributed shared
+//     memory, ~440 cycles), and a pass ends with a cluster barrier (~500 cycles): these two are what
+//     a pass takes, whatever the level;
+//   * restriction and prolongation read the planes they need wherever these are;
+//   * every CTA gathers the coarsest right-hand side and computes some of the inverse's rows.
+// A neighbour beyond a wall is another cell of that colour, or a zero of the row of zeros before and after each
+// colour's cells, with a zero coefficient: an update has no wall tests, the product is a zero.
+// The arithmetic of a cell is that of the kernels of the larger levels, in their order, so the
+// results are those of a launch per pass.  What it measures: launch_tail.
 // ---------------------------------------------------------------------------
-// threads of the descent (its residual-restriction needs more registers) and of the ascent
-constexpr int kTailDownThreads = 512, kTailUpThreads = 1024;
-
 template <typename T>
-__device__ void tail_colour(const TailLevel<T> &v, int colour)
+__global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs<T> a)
 {
-    const int hx = (v.nx + 1) / 2, total = hx * v.ny * v.nz;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int jk = (int)fdiv(t, v.fhx), k = (int)fdiv(jk, v.fny);
-        const int u = t - jk * hx, j = jk - k * v.ny;
-        const int i = 2 * u + ((j + k + colour) & 1);
-        if (i < v.nx && ck_cell(((long long)k * v.ny + j) * v.nx + i, i, j, k, v.nx, v.ny, v.nz, CK_TAIL))
-            smooth_cell<T, true>(i, j, k, v.nx, v.ny, v.nz, v.h2, v.L, v.L.b, v.L.p);
-    }
-    __syncthreads();
-}
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *const sm = reinterpret_cast<T *>(smem_raw);
+    const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
+    const int tid = threadIdx.x, nthr = kTailThreads, top = a.nlev - 1;
 
-template <typename T>
-__device__ void tail_restrict(const TailLevel<T> &f, T *bc)
-{
-    const int NX = f.nx / 2, NY = f.ny / 2, total = NX * NY * (f.nz / 2);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int JK = (int)fdiv(t, f.fcx), K = (int)fdiv(JK, f.fcy);
-        const int I = t - JK * NX, J = JK - K * NY;
-        restrict_box<T, false>(I, J, K, f.nx, f.ny, f.nz, f.ih2, f.L, f.L.b, f.L.p, bc, 0);
-    }
-    __syncthreads();
-}
-
-template <typename T>
-__device__ void tail_prolong(const TailLevel<T> &f, const T *ec, bool red)
-{
-    const int NX = f.nx / 2, NY = f.ny / 2, NZ = f.nz / 2, total = NX * NY * NZ;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int JK = (int)fdiv(t, f.fcx), K = (int)fdiv(JK, f.fcy);
-        const int I = t - JK * NX, J = JK - K * NY;
-        if (red) {
-            prolong_red<T, false>(I, J, K, f.nx, f.ny, f.nz, ec, f.L.dinv, f.L.p);
-            continue;
+    // the slabs of every level: p = 0, faces and inverse diagonals, the top level's b
+    for (int l = 0; l < top; l++) {
+        const TailLevel<T> &v = a.lev[l];
+        const int z0 = rank * v.P, nk = max(0, min(v.nz - z0, v.P));
+        const unsigned hx = v.nx / 2, hxy = hx * v.ny, H = v.P * hxy + hx, HZ = H + hxy;
+        const unsigned total = (unsigned)nk * 2 * hxy, plane = 2 * hxy;
+        const size_t g0 = (size_t)z0 * plane;
+        for (unsigned c = tid; c < 2 * H + hx; c += nthr) sm[v.op - hx + c] = T(0);
+        for (unsigned c = tid; c < total + plane; c += nthr) {  // the plane above for its low z-faces
+            const bool own = c < total;
+            if (!own && (nk == 0 || z0 + nk >= v.nz)) break;
+            if (!MG_CK(g0 + c, g0 + c, (long long)plane * v.nz, CK_TAIL)) break;
+            const unsigned row = fdiv(c, v.fnx), i = c - row * v.nx, kl = fdiv(row, v.fny), j = row - kl * v.ny;
+            const unsigned q = (i + j + kl + z0) & 1u, m = c >> 1;
+            sm[v.oz + q * HZ + m] = v.L.bz[g0 + c];
+            if (own) {
+                sm[v.ox + q * H + m] = v.L.bx[g0 + c];
+                sm[v.oy + q * H + m] = v.L.by[g0 + c];
+                sm[v.od + q * H + m] = v.L.dinv[g0 + c];
+                if (l == 0) sm[v.ob + q * H + m] = v.L.b[g0 + c];
+            }
         }
-        T corr[2][2][2];
-        prolong_corr<T>(I, J, K, NX, NY, NZ, ec, corr);
+    }
+    cl.sync();
+
+    // n sweeps on level v, colour `first` first; zero: the level's p is zero (a first red pass reads
+    // no neighbour)
+    auto sweeps = [&](const TailLevel<T> &v, int n, unsigned first, bool zero) {
+        if (n == 0) return;
+        const int z0 = rank * v.P, nk = max(0, min(v.nz - z0, v.P));
+        const unsigned hx = v.nx / 2, hxy = hx * v.ny, H = v.P * hxy + hx, HZ = H + hxy, total = nk * hxy;
+        T *const p = sm + v.op;
+        const T *const below = rank > 0 ? cl.map_shared_rank(p, rank - 1) + (v.P - 1) * hxy : p;
+        const T *const above = rank + 1 < ncta ? cl.map_shared_rank(p, rank + 1) : p;
+        T fxl[kTailCells][2], fxh[kTailCells][2], fyl[kTailCells][2], fyh[kTailCells][2], fzl[kTailCells][2],
+            fzh[kTailCells][2], fd[kTailCells][2], fb[kTailCells][2];
+        const T *zl[kTailCells], *zh[kTailCells];  // the planes below and above (colour 0)
+        unsigned odd[kTailCells];                   // (j + k) & 1
 #pragma unroll
-        for (int dz = 0; dz < 2; dz++)
+        for (int e = 0; e < kTailCells; e++) {
+            const unsigned t = tid + e * nthr;
+            odd[e] = 0;
+            zl[e] = zh[e] = p;
+            if (t >= total) continue;
+            const unsigned row = fdiv(t, v.fhx), u = t - row * hx, kl = fdiv(row, v.fny), j = row - kl * v.ny;
+            const unsigned k = z0 + kl, t0 = t - kl * hxy;
+            odd[e] = (j + k) & 1u;
+            zl[e] = k == 0 ? p + t : (kl > 0 ? p + t - hxy : below + t0);
+            zh[e] = k + 1 == (unsigned)v.nz ? p + t : (kl + 1 < (unsigned)v.P ? p + t + hxy : above + t0);
 #pragma unroll
-            for (int dy = 0; dy < 2; dy++)
+            for (unsigned q = 0; q < 2; q++) {
+                const unsigned off = odd[e] ^ q, i = 2 * u + off, o = q ^ 1u;
+                fxl[e][q] = i > 0 ? sm[v.ox + q * H + t] : T(0);
+                fxh[e][q] = i + 1 < (unsigned)v.nx ? sm[v.ox + o * H + t + off] : T(0);
+                fyl[e][q] = j > 0 ? sm[v.oy + q * H + t] : T(0);
+                fyh[e][q] = j + 1 < (unsigned)v.ny ? sm[v.oy + o * H + t + hx] : T(0);
+                fzl[e][q] = k > 0 ? sm[v.oz + q * HZ + t] : T(0);
+                fzh[e][q] = k + 1 < (unsigned)v.nz ? sm[v.oz + o * HZ + t + hxy] : T(0);
+                fd[e][q] = sm[v.od + q * H + t];
+                fb[e][q] = sm[v.ob + q * H + t];
+            }
+        }
+        auto pass = [&](auto colour) {
+            constexpr unsigned q = decltype(colour)::value, o = q ^ 1u;
 #pragma unroll
-                for (int dx = 0; dx < 2; dx++) {
-                    const size_t c = ((size_t)(2 * K + dz) * f.ny + (2 * J + dy)) * f.nx + 2 * I + dx;
-                    if (!MG_CK(c, c, (long long)f.nx * f.ny * f.nz, CK_TAIL)) continue;
-                    if (!zero_bits(f.L.dinv[c])) f.L.p[c] = f.L.p[c] + corr[dz][dy][dx];
+            for (int e = 0; e < kTailCells; e++) {
+                const unsigned t = tid + e * nthr;
+                if (t >= total) break;
+                T s = T(0);
+                if (!zero) {
+                    const T *const ot = p + o * H + t, *const ox = ot + (odd[e] ^ q);
+                    s = fma(fxl[e][q], ox[-1], s);
+                    s = fma(fxh[e][q], ox[0], s);
+                    s = fma(fyl[e][q], *(ot - hx), s);
+                    s = fma(fyh[e][q], *(ot + hx), s);
+                    s = fma(fzl[e][q], zl[e][o * H], s);
+                    s = fma(fzh[e][q], zh[e][o * H], s);
                 }
-    }
-    __syncthreads();
-}
-
-// descent: on each level but the coarsest, zero p (below the first), nu1 sweeps red then
-// black, residual restricted to the next level's b
-template <typename T>
-__global__ void __launch_bounds__(kTailDownThreads) k_tail_down(TailArgs<T> a)
-{
-    for (int l = 0; l < a.nlev - 1; l++) {
-        const TailLevel<T> v = a.lev[l];
-        if (l > 0 || a.zero0) {
-            const int n = v.nx * v.ny * v.nz;
-            for (int t = threadIdx.x; t < n; t += blockDim.x) v.L.p[t] = T(0);
-            __syncthreads();
+                p[q * H + t] = fd[e][q] * fma(-v.h2, fb[e][q], s);
+            }
+            zero = false;
+            cl.sync();
+        };
+        for (int it = 0; it < n; it++) {
+            if (first == 0) {
+                pass(std::integral_constant<unsigned, 0>{});
+                pass(std::integral_constant<unsigned, 1>{});
+            } else {
+                pass(std::integral_constant<unsigned, 1>{});
+                pass(std::integral_constant<unsigned, 0>{});
+            }
         }
-        for (int it = 0; it < a.nu1; it++) {
-            tail_colour<T>(v, 0);
-            tail_colour<T>(v, 1);
-        }
-        tail_restrict<T>(v, a.lev[l + 1].L.b);
-    }
-}
+    };
+    // base of plane k of an array at offset o of level v, in the shared memory that holds it
+    auto plane_of = [&](const TailLevel<T> &v, unsigned o, unsigned k, unsigned stride) {
+        const unsigned r = fdiv(k, v.fP);
+        return cl.map_shared_rank(sm + o, r) + (k - r * v.P) * stride;
+    };
+    // where cell (I, J) of a plane of level v sits (the coarsest level is kept in natural order)
+    auto slot = [&](const TailLevel<T> &v, bool last, unsigned I, unsigned J, unsigned K) {
+        const unsigned hx = v.nx / 2;
+        return last ? J * v.nx + I : ((I + J + K) & 1u) * (v.P * hx * v.ny + hx) + J * hx + (I >> 1);
+    };
 
-// ascent: from the level above the coarsest up, prolong the coarser correction, nu2 sweeps
-// black then red
-template <typename T>
-__global__ void __launch_bounds__(kTailUpThreads) k_tail_up(TailArgs<T> a)
-{
-    for (int l = a.nlev - 2; l >= 0; l--) {
-        const TailLevel<T> v = a.lev[l];
-        tail_prolong<T>(v, a.lev[l + 1].L.p, a.nu2 >= 1);
-        for (int it = 0; it < a.nu2; it++) {
-            tail_colour<T>(v, 1);
-            tail_colour<T>(v, 0);
+    // descent: nu1 sweeps red then black, restriction (restrict_box)
+    for (int l = 0; l < top; l++) {
+        const TailLevel<T> &v = a.lev[l], &w = a.lev[l + 1];
+        sweeps(v, a.nu1, 0, true);
+        const bool last = l + 1 == top;
+        const unsigned hx = v.nx / 2, hxy = hx * v.ny, H = v.P * hxy + hx, HZ = H + hxy;
+        const int Z0 = rank * w.P, nK = max(0, min(w.nz - Z0, w.P));
+        const unsigned NX = w.nx, NY = w.ny, total = (unsigned)nK * NX * NY, stride_w = last ? NX * NY : NX / 2 * NY;
+        for (unsigned t = tid; t < total; t += nthr) {
+            const unsigned row = fdiv(t, w.fnx), I = t - row * NX, Kl = fdiv(row, w.fny), J = row - Kl * NY;
+            const unsigned K = Z0 + Kl;
+            T s = T(0), sb = T(0);
+#pragma unroll
+            for (unsigned dk = 0; dk < 2; dk++) {
+                const unsigned k = 2 * K + dk;
+                const T *const p = plane_of(v, v.op, k, hxy), *const b = plane_of(v, v.ob, k, hxy);
+                const T *const X = plane_of(v, v.ox, k, hxy), *const Y = plane_of(v, v.oy, k, hxy);
+                const T *const Z = plane_of(v, v.oz, k, hxy) + (dk ? hxy : 0);
+                const bool hz = dk ? k + 1 < (unsigned)v.nz : k > 0;
+                const T *const pz = hz ? plane_of(v, v.op, dk ? k + 1 : k - 1, hxy) : p;
+#pragma unroll
+                for (unsigned dj = 0; dj < 2; dj++) {
+                    const unsigned j = 2 * J + dj, q = dj ^ dk, e = j * hx + I;  // q: colour of the even cell
+                    const unsigned E = q * H + e, O = (q ^ 1u) * H + e;
+                    const T pe = p[E], po = p[O];
+                    if (I > 0) s = fma(X[E], p[O - 1] - pe, s);
+                    if (I + 1 < hx) s = fma(X[E + 1], p[E + 1] - po, s);
+                    if (dj ? j + 1 < (unsigned)v.ny : j > 0) {
+                        const T fe = dj ? Y[O + hx] : Y[E], fo = dj ? Y[E + hx] : Y[O];
+                        s = fma(fe, (dj ? p[O + hx] : p[O - hx]) - pe, s);
+                        s = fma(fo, (dj ? p[E + hx] : p[E - hx]) - po, s);
+                    }
+                    if (hz) {
+                        const unsigned ZE = q * HZ + e, ZO = (q ^ 1u) * HZ + e;
+                        s = fma(Z[dk ? ZO : ZE], pz[O] - pe, s);
+                        s = fma(Z[dk ? ZE : ZO], pz[E] - po, s);
+                    }
+                    sb += b[E] + b[O];
+                }
+            }
+            sm[w.ob + Kl * stride_w + slot(w, last, I, J, K)] = T(0.125) * fma(-s, v.ih2, sb);
+        }
+        cl.sync();
+    }
+
+    // the coarsest grid: e = M b, a row per warp (k_coarse_solve)
+    {
+        const TailLevel<T> &w = a.lev[top];
+        const unsigned NXY = w.nx * w.ny, n = NXY * w.nz;
+        double *const sb = reinterpret_cast<double *>(smem_raw + a.sb_bytes);
+        for (unsigned t = tid; t < n; t += nthr) {
+            const unsigned K = fdiv(fdiv(t, w.fnx), w.fny);
+            sb[t] = (double)plane_of(w, w.ob, K, NXY)[t - K * NXY];
+        }
+        __syncthreads();
+        const unsigned warps = nthr / 32, lane = tid & 31;
+        for (unsigned r = rank * warps + tid / 32; r < n; r += ncta * warps) {
+            if (!MG_CK((long long)r * n, (long long)r * n + n - 1, (long long)n * n, CK_COARSE_SOLVE)) continue;
+            const double *row = a.M + (size_t)r * n;
+            double s = 0.0;
+            for (unsigned q = lane; q < n; q += 32) s = fma(row[q], sb[q], s);
+            s = warp_sum(s);
+            const unsigned K = fdiv(fdiv(r, w.fnx), w.fny);
+            if (lane == 0) plane_of(w, w.op, K, NXY)[r - K * NXY] = (T)s;
+        }
+        cl.sync();
+    }
+
+    // ascent: prolongation (of the red cells alone where a black pass follows), nu2 sweeps black then red
+    for (int l = top - 1; l >= 0; l--) {
+        const TailLevel<T> &v = a.lev[l], &w = a.lev[l + 1];
+        const bool last = l + 1 == top;
+        const int z0 = rank * v.P, nk = max(0, min(v.nz - z0, v.P));
+        const unsigned hx = v.nx / 2, hxy = hx * v.ny, H = v.P * hxy + hx, total = nk * hxy;
+        const unsigned stride_w = last ? w.nx * w.ny : w.nx / 2 * w.ny;
+        for (unsigned q = 0; q < (a.nu2 >= 1 ? 1u : 2u); q++)
+            for (unsigned t = tid; t < total; t += nthr) {
+                const unsigned row = fdiv(t, v.fhx), u = t - row * hx, kl = fdiv(row, v.fny), j = row - kl * v.ny;
+                const unsigned k = z0 + kl, i = 2 * u + ((j + k + q) & 1u);
+                // parent and the neighbour on the cell's side, clamped at the walls
+                auto next = [](unsigned f, int n) {
+                    return (f & 1u) ? min((f >> 1) + 1, (unsigned)n - 1) : ((f >> 1) ? (f >> 1) - 1 : 0u);
+                };
+                const unsigned Ks[2] = {k >> 1, next(k, w.nz)}, Js[2] = {j >> 1, next(j, w.ny)},
+                               Is[2] = {i >> 1, next(i, w.nx)};
+                const T wt[2] = {T(0.75), T(0.25)};
+                T s = T(0);
+#pragma unroll
+                for (int z = 0; z < 2; z++) {
+                    const T *const e = plane_of(w, w.op, Ks[z], stride_w);
+#pragma unroll
+                    for (int y = 0; y < 2; y++)
+#pragma unroll
+                        for (int x = 0; x < 2; x++)
+                            s = fma(wt[z] * wt[y] * wt[x], e[slot(w, last, Is[x], Js[y], Ks[z])], s);
+                }
+                if (!zero_bits(sm[v.od + q * H + t])) sm[v.op + q * H + t] += s;
+            }
+        cl.sync();
+        sweeps(v, a.nu2, 1, false);
+    }
+
+    // the top level's correction (every remote read of this CTA's memory lies before the last barrier)
+    {
+        const TailLevel<T> &v = a.lev[0];
+        const int z0 = rank * v.P, nk = max(0, min(v.nz - z0, v.P));
+        const unsigned hx = v.nx / 2, hxy = hx * v.ny, H = v.P * hxy + hx, total = (unsigned)nk * 2 * hxy;
+        const size_t g0 = (size_t)z0 * 2 * hxy;
+        for (unsigned c = tid; c < total; c += nthr) {
+            const unsigned row = fdiv(c, v.fnx), i = c - row * v.nx, kl = fdiv(row, v.fny), j = row - kl * v.ny;
+            if (!MG_CK(g0 + c, g0 + c, (long long)2 * hxy * v.nz, CK_TAIL)) break;
+            v.L.p[g0 + c] = sm[v.op + ((i + j + kl + z0) & 1u) * H + (c >> 1)];
         }
     }
 }
@@ -3063,26 +3214,72 @@ cudaError_t launch_coarse_solve(int n, const double *M, const T *b, T *e, cudaSt
                                                                                                                 e);
     return cudaGetLastError();
 }
+// a launch of k_tail on a cluster (of more than 8 CTAs by opt-in)
 template <typename T>
-cudaError_t launch_tail_down(const TailArgs<T> &a, cudaStream_t s)
+cudaError_t tail_config(int ctas, size_t smem, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at)
 {
-    if (a.nlev < 2 || a.nlev > kTailMaxLevels) return cudaErrorInvalidValue;
-    note_launch();
-    k_tail_down<T><<<1, kTailDownThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && ctas > 8)
+        e = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cfg = cudaLaunchConfig_t{};
+    at = cudaLaunchAttribute{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return e;
 }
+
+// CTAs of the largest cluster (16, else 8) that the current device holds with kTailSmem bytes each, 0 if
+// neither: a property of the device, asked once for each (the query takes some 80 us)
 template <typename T>
-cudaError_t launch_tail_up(const TailArgs<T> &a, cudaStream_t s)
+int tail_ctas()
 {
-    if (a.nlev < 2 || a.nlev > kTailMaxLevels) return cudaErrorInvalidValue;
-    note_launch();
-    k_tail_up<T><<<1, kTailUpThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];  // 1 + the answer
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < kDevices && known[dev].load() > 0) return known[dev].load() - 1;
+    int n = 0;
+    for (int ctas : {16, 8}) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        int clusters = 0;
+        if (tail_config<T>(ctas, kTailSmem, cfg, at) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_tail<T>, &cfg) == cudaSuccess && clusters >= 1) {
+            n = ctas;
+            break;
+        }
+        cudaGetLastError();
+    }
+    if (dev < kDevices) known[dev].store(n + 1);
+    return n;
 }
-template cudaError_t launch_tail_down<double>(const TailArgs<double> &, cudaStream_t);
-template cudaError_t launch_tail_down<float>(const TailArgs<float> &, cudaStream_t);
-template cudaError_t launch_tail_up<double>(const TailArgs<double> &, cudaStream_t);
-template cudaError_t launch_tail_up<float>(const TailArgs<float> &, cudaStream_t);
+template int tail_ctas<double>();
+template int tail_ctas<float>();
+
+// Coarse-grid correction below a grid, us (a launch per pass -> this kernel -> one CTA with its fields in
+// L1, two launches and the exact solve between, as it was): 32^3 FP32 35 -> 21 (35), FP64 45 -> 27 (86);
+// 64^3 FP32 47 -> 35 (50), FP64 64 -> 48 (111); 192x160x224 FP32 92 -> 87 (96).  With a coarsest grid of
+// 512 cells, whose inverse 16 SMs apply in the time of the launches saved: 116 -> 116 (125) FP32.
+template <typename T>
+cudaError_t launch_tail(const TailArgs<T> &a, cudaStream_t s)
+{
+    if (a.nlev < 2 || a.nlev > kTailMaxLevels || a.ctas < 1 || a.smem > kTailSmem) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    const cudaError_t e = tail_config<T>(a.ctas, a.smem, cfg, at);
+    if (e != cudaSuccess) return e;
+    cfg.stream = s;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, k_tail<T>, a);
+}
+template cudaError_t launch_tail<double>(const TailArgs<double> &, cudaStream_t);
+template cudaError_t launch_tail<float>(const TailArgs<float> &, cudaStream_t);
 
 template cudaError_t launch_coarse_solve<double>(int, const double *, const double *, double *, cudaStream_t);
 template cudaError_t launch_coarse_solve<float>(int, const double *, const float *, float *, cudaStream_t);

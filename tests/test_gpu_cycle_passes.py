@@ -68,3 +68,29 @@ def test_continued_cycles_are_the_single_ones(mgp, shape):
     q = O.remove_mean(host(q), lab, nc)
     assert st.cycles == 3
     assert np.abs(host(p) - q).max() <= 1e-13 * np.abs(q).max()
+
+
+# first tail level (half the grid): planes that do and do not deal out evenly over 16 CTAs, fewer planes
+# than CTAs, more cells per CTA than threads, the largest tail (8192 cells) and one cell more per axis,
+# a coarsest grid of an odd size, one above the size the tail solves
+TAIL_SHAPES = [(32, 32, 40), (16, 16, 144), (64, 64, 16), (48, 80, 24), (32, 32, 64), (36, 32, 64), (20, 24, 28),
+               (44, 44, 44)]
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (0, 1), (1, 0)])
+@pytest.mark.parametrize("shape", TAIL_SHAPES)
+def test_tail_slabs_identical_to_launches(mgp, shape, nu):
+    """The tail's cluster, whichever way the planes fall on its CTAs, gives the V-cycles of a launch
+    per pass bit for bit (the same operations in the same order)."""
+    case = synth.small_case(*shape, solid="ellipsoid", seed=52)
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    rhs = dev(case.rhs)
+    for prec in ("fp64", "mixed"):
+        out = []
+        for tail in (0, 1):
+            ctx = mgp.Context(beta, case.h, prec=prec, coarse_tail=tail, nu1=nu[0], nu2=nu[1], coarse_max_cells=2048)
+            p = torch.zeros_like(rhs)
+            for _ in range(2):
+                ctx.vcycle(rhs, p)
+            out.append(p)
+        assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1]), prec
