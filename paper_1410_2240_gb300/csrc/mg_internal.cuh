@@ -26,10 +26,9 @@ struct LevelArrays {
     T *p = nullptr;                                  // correction (levels >= 1)
 };
 
-// Number of CTAs of the grid-stride vector and reduction kernels (16 per SM on 152 SMs,
-// enough loads in flight to keep HBM busy).  A reduction's partials buffer holds 2 * kRedBlocks
-// doubles and, after them, the counter of the blocks that have finished (kRedPartials doubles in
-// all, the counter zero between reductions).
+// Blocks of a grid-stride reduction at most (red_grid and vec_grid in mg_kernels.cu give the number).  A
+// reduction's partials buffer holds 2 * kRedBlocks doubles and, after them, the counter of the blocks that
+// have finished (kRedPartials doubles in all, the counter zero between reductions).
 constexpr int kRedBlocks = 2432;
 constexpr int kRedPartials = 2 * kRedBlocks + 2;
 constexpr int kRedThreads = 256;

@@ -35,22 +35,43 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sum over the block; the result is valid in thread 0.  NT = blockDim.x.
-template <int NT>
-__device__ double block_sum(double v)
+// Sums of a and b over the block (NT = blockDim.x threads), valid in thread 0.  An FP64 addition holds
+// a scheduler's FP64 unit for some 79 cycles whatever the lanes it is for, so the sums are taken with
+// few warp-wide additions: every thread stores its pair, one warp per sum adds the warps' values lane by
+// lane and then its own lanes (7 + 5 additions a sum for 256 threads, 45 when every warp first added its
+// own lanes: 12 us of a 256^3 pass, the whole time of a 128^3 one).
+template <int NT, bool TWO = true>
+__device__ __forceinline__ void block_sum2(double &a, double &b)
 {
-    __shared__ double sh[NT / 32];
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
+    constexpr int W = NT / 32;
+    __shared__ double sh[2][NT];
+    sh[0][threadIdx.x] = a;
+    if (TWO) sh[1][threadIdx.x] = b;
     __syncthreads();
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     double r = 0.0;
-    if (w == 0) {
-        r = (l < NT / 32) ? sh[l] : 0.0;
-        r = warp_sum(r);
+    if (w < (TWO ? 2 : 1)) {
+        double v[W];
+#pragma unroll
+        for (int k = 0; k < W; k++) v[k] = sh[w][32 * k + l];
+#pragma unroll
+        for (int o = W / 2; o > 0; o /= 2)
+#pragma unroll
+            for (int k = 0; k < o; k++) v[k] += v[k + o];
+        r = warp_sum(v[0]);
+        if (TWO && w == 1 && l == 0) sh[1][0] = r;  // (lane 0 alone read that word)
     }
     __syncthreads();
-    return r;
+    a = r;
+    if (TWO) b = sh[1][0];
+    __syncthreads();
+}
+template <int NT>
+__device__ __forceinline__ double block_sum(double v)
+{
+    double none = 0.0;
+    block_sum2<NT, false>(v, none);
+    return v;
 }
 
 // A scalar every thread of a block needs, computed by thread 0 and shared: FP64 divisions and
@@ -75,8 +96,7 @@ __global__ void k_finish2(const double *__restrict__ partials, int nblocks, doub
         a += partials[2 * i];
         b += partials[2 * i + 1];
     }
-    a = block_sum<kRedThreads>(a);
-    b = block_sum<kRedThreads>(b);
+    block_sum2<kRedThreads>(a, b);
     if (threadIdx.x == 0) {
         if (slot0 >= 0) dscal[slot0] = a;
         if (slot1 >= 0) dscal[slot1] = b;
@@ -116,8 +136,7 @@ __device__ bool reduce_finish(double a, double b, double *partials, double *dsca
             y += y1;
         }
     }
-    x = block_sum<kRedThreads>(x);
-    y = block_sum<kRedThreads>(y);
+    block_sum2<kRedThreads>(x, y);
     if (threadIdx.x == 0) {
         if (slot0 >= 0) dscal[slot0] = x;
         if (slot1 >= 0) dscal[slot1] = y;
@@ -1678,10 +1697,10 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
 // ---------------------------------------------------------------------------
 __global__ void k_count_live(unsigned n, const double *__restrict__ dinv, double *__restrict__ partials, double *dscal)
 {
-    double a = 0.0;
+    unsigned a = 0;  // counted in integers: the FP64 unit would bound the pass
     for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x)
-        a += pos_bits(dinv[idx]) ? 1.0 : 0.0;
-    reduce_finish(block_sum<kRedThreads>(a), 0.0, partials, dscal, S_NLIVE, -1);
+        a += pos_bits(dinv[idx]) ? 1u : 0u;
+    reduce_finish(block_sum<kRedThreads>((double)a), 0.0, partials, dscal, S_NLIVE, -1);
 }
 
 // pass 1 of the rhs preparation: sum of rhs over live cells
@@ -1728,8 +1747,7 @@ __global__ void k_resid_norm(int nx, int ny, int nz, double ih2, LevelArrays<dou
         rr += r * r;
         if (pos_bits(L.dinv[idx])) sp += p[idx];
     }
-    rr = block_sum<kRedThreads>(rr);
-    sp = block_sum<kRedThreads>(sp);
+    block_sum2<kRedThreads>(rr, sp);
     reduce_finish(rr, sp, partials, dscal, S_RR, S_SUM_P);
 }
 
@@ -1762,8 +1780,7 @@ __global__ void k_resid_cast(int nx, int ny, int nz, double ih2, LevelArrays<dou
         const size_t slot = half ? split_slot(idx, (j + k) & 1, half) : idx;
         if (MG_CK(slot, slot, (long long)n, CK_SPLIT_SLOT)) r32[slot] = narrow(r * inv_scale);
     }
-    rr = block_sum<kRedThreads>(rr);
-    sp = block_sum<kRedThreads>(sp);
+    block_sum2<kRedThreads>(rr, sp);
     // the last block also sets the next scale: the RMS of this residual over the live cells (1 if 0)
     if (reduce_finish(rr, sp, partials, dscal, S_RR, S_SUM_P) && threadIdx.x == 0 && scale_out >= 0) {
         const double rms = sqrt(dscal[S_RR] / dscal[S_NLIVE]);
@@ -2499,8 +2516,7 @@ __global__ void k_pcg_resid(int nx, int ny, int nz, double ih2, LevelArrays<doub
         run(BoolTag<true>{});
     else
         run(BoolTag<false>{});
-    rr = block_sum<kRedThreads>(rr);
-    sp = block_sum<kRedThreads>(sp);
+    block_sum2<kRedThreads>(rr, sp);
     reduce_finish(rr, sp, partials, dscal, S_RR, S_SUM_P);
 }
 
@@ -2517,9 +2533,8 @@ __global__ void k_pcg_dots(unsigned n, const double *__restrict__ r, const Z *__
         a = fma(rv, (double)z[idx], a);
         if (zo) c = fma(rv, (double)zo[idx], c);
     }
-    a = block_sum<kRedThreads>(a) * sz;
-    c = block_sum<kRedThreads>(c) * so;
-    reduce_finish(a, c, partials, dscal, S_RZN, S_RZO);
+    block_sum2<kRedThreads>(a, c);
+    reduce_finish(a * sz, c * so, partials, dscal, S_RZN, S_RZO);
 }
 
 // Mixed-precision variant: <r, z> = sr sz <r32, e32> from the FP32 copy r32 = r / sr that the
@@ -2556,8 +2571,9 @@ __global__ void k_pcg_dots32(unsigned n, const float *__restrict__ r32, const fl
         a += widen(r32[idx] * z[idx]);
         if (zo) c += widen(r32[idx] * zo[idx]);
     }
-    a = block_sum<kRedThreads>(a) * sr * dscal[sz_slot];
-    c = block_sum<kRedThreads>(c) * (so_slot >= 0 ? sr * dscal[so_slot] : 0.0);
+    block_sum2<kRedThreads>(a, c);
+    a = a * sr * dscal[sz_slot];
+    c = c * (so_slot >= 0 ? sr * dscal[so_slot] : 0.0);
     reduce_finish(a, c, partials, dscal, S_RZN, S_RZO);
 }
 
@@ -2932,8 +2948,7 @@ __global__ void k_comp_center(unsigned n, const double *__restrict__ v, const in
         out[idx] = o;
         a += o * o;
     }
-    a = block_sum<kRedThreads>(a);
-    b = block_sum<kRedThreads>(b);
+    block_sum2<kRedThreads>(a, b);
     if (threadIdx.x == 0) {
         partials[2 * blockIdx.x] = a;
         partials[2 * blockIdx.x + 1] = b;
@@ -2976,10 +2991,24 @@ inline dim3 row_grid2(int threads_x, int ny, int nz)
     return dim3((unsigned)((threads_x + b.x - 1) / b.x), (unsigned)((ny + b.y - 1) / b.y), (unsigned)nz);
 }
 
+// Blocks of the grid-stride reductions: at most five per SM, so that the grid is one wave (the operator
+// of the CG holds six blocks per SM by its registers) and its end reads few partials, and on small
+// grids at least four cells per thread beyond two blocks per SM.  CG operator + update + dots and
+// direction, mixed: 241 + 182 + 100 us at 256^3 with 16 blocks per SM, 241 + 177 + 92 us with five,
+// 238 + 175 + 96 with four; 128^3: 45 + 38 + 36 us with 16, 39 + 31 + 26 with five; 64^3: 14 + 15 + 18 us with up to 16,
+// 12 + 14 + 16 with two.
 inline unsigned red_grid(size_t n)
 {
-    size_t b = (n + kRedThreads - 1) / kRedThreads;
-    return (unsigned)(b < (size_t)kRedBlocks ? (b ? b : 1) : kRedBlocks);
+    const size_t b = (n + kRedThreads - 1) / kRedThreads, sm = 152;
+    return (unsigned)std::max<size_t>(1, std::min({b, std::max(2 * sm, b / 4), 5 * sm}));
+}
+// Blocks of the vector passes without a reduction and of the FP64 CG's dots and direction, which
+// stream and have no FP64 arithmetic to hide latency behind: eight per SM (FP64 CG vectors at 256^3: 129 us, 138 us with
+// five, 133 us with 16).
+inline unsigned vec_grid(size_t n)
+{
+    const size_t b = (n + kRedThreads - 1) / kRedThreads;
+    return (unsigned)std::max<size_t>(1, std::min<size_t>(b, 8 * 152));
 }
 
 }  // namespace
@@ -2999,7 +3028,7 @@ cudaError_t launch_face_coeffs(Dims d, const double *phi, const uint8_t *solid, 
 cudaError_t launch_jacobi(size_t n, double scale, const double *dinv, const double *r, double *z, cudaStream_t s)
 {
     note_launch();
-    k_jacobi<<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, scale, dinv, r, z);
+    k_jacobi<<<vec_grid(n), kRedThreads, 0, s>>>((unsigned)n, scale, dinv, r, z);
     return cudaGetLastError();
 }
 
@@ -3294,9 +3323,9 @@ cudaError_t launch_components(Dims d, const double *dinv, const double *bx, cons
     note_launch();
     k_cc_rows<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(d.nx, d.ny, d.nz, dinv, bx, label);
     note_launch();
-    k_cc_merge<<<red_grid(n), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, bx, by, bz, label, ctr + 1);
+    k_cc_merge<<<vec_grid(n), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, bx, by, bz, label, ctr + 1);
     note_launch();
-    k_cc_flatten<<<red_grid(n), kRedThreads, 0, s>>>(n, label, ctr, ctr + 1);
+    k_cc_flatten<<<vec_grid(n), kRedThreads, 0, s>>>(n, label, ctr, ctr + 1);
     return cudaGetLastError();
 }
 
@@ -3306,7 +3335,7 @@ cudaError_t launch_component_roots(size_t n, const int *label, int *roots, unsig
     cudaError_t e = cudaMemsetAsync(slot, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     note_launch();
-    k_cc_roots<<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, label, roots, slot, cap);
+    k_cc_roots<<<vec_grid(n), kRedThreads, 0, s>>>((unsigned)n, label, roots, slot, cap);
     return cudaGetLastError();
 }
 
@@ -3314,7 +3343,7 @@ cudaError_t launch_component_compact(size_t n, int *label, const int *sorted_roo
                                      double *part, cudaStream_t s)
 {
     note_launch();
-    k_cc_compact<<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, label, sorted_roots, ncomp);
+    k_cc_compact<<<vec_grid(n), kRedThreads, 0, s>>>((unsigned)n, label, sorted_roots, ncomp);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_comp_sums(n, nullptr, label, ncomp, cnt, part, s);
@@ -3337,7 +3366,7 @@ cudaError_t launch_comp_sums(size_t n, const double *v, const int *comp, int nco
     if (e != cudaSuccess) return e;
     const unsigned threads = (unsigned)((n + kCcChunk - 1) / kCcChunk);
     note_launch();
-    k_comp_sums<<<red_grid(threads), kRedThreads, 0, s>>>((unsigned)n, v, comp, sums);
+    k_comp_sums<<<vec_grid(threads), kRedThreads, 0, s>>>((unsigned)n, v, comp, sums);
     return cudaGetLastError();
 }
 
@@ -3386,7 +3415,7 @@ cudaError_t launch_resid_norm(Dims d, double ih2, const LevelArrays<double> &L, 
 cudaError_t launch_sub_mean_p(Dims d, const double *dinv, double *p, const double *dscal, cudaStream_t s)
 {
     note_launch();
-    k_sub_mean_p<<<red_grid(d.n()), kRedThreads, 0, s>>>((unsigned)d.n(), dinv, p, dscal);
+    k_sub_mean_p<<<vec_grid(d.n()), kRedThreads, 0, s>>>((unsigned)d.n(), dinv, p, dscal);
     return cudaGetLastError();
 }
 
@@ -3409,14 +3438,14 @@ cudaError_t launch_resid_cast(Dims d, double ih2, const LevelArrays<double> &L, 
 cudaError_t launch_to_f32_layout(size_t n, const double *src, float *dst, cudaStream_t s, Split sp)
 {
     note_launch();
-    k_to_f32_layout<<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, src, dst, sp);
+    k_to_f32_layout<<<vec_grid(n), kRedThreads, 0, s>>>((unsigned)n, src, dst, sp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_from_f32_layout(size_t n, const float *src, double *dst, cudaStream_t s, Split sp)
 {
     note_launch();
-    k_from_f32_layout<<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, src, dst, sp);
+    k_from_f32_layout<<<vec_grid(n), kRedThreads, 0, s>>>((unsigned)n, src, dst, sp);
     return cudaGetLastError();
 }
 
@@ -3425,7 +3454,7 @@ cudaError_t launch_accumulate(Dims d, const double *dinv, const float *e32, doub
 {
     note_launch();
     (void)dinv;
-    k_accumulate<<<red_grid(d.n()), kRedThreads, 0, s>>>((unsigned)d.n(), e32, p, dscal, scale_slot, sp);
+    k_accumulate<<<vec_grid(d.n()), kRedThreads, 0, s>>>((unsigned)d.n(), e32, p, dscal, scale_slot, sp);
     return cudaGetLastError();
 }
 
@@ -3470,7 +3499,7 @@ cudaError_t launch_rk_combine(size_t n, const LevelArrays<double> &a, const Leve
                               const LevelArrays<double> &r, double dt, const LevelArrays<double> &out, cudaStream_t s)
 {
     note_launch();
-    k_rk_combine<<<red_grid(n), kRedThreads, 0, s>>>(n, a, b, r, dt, out);
+    k_rk_combine<<<vec_grid(n), kRedThreads, 0, s>>>(n, a, b, r, dt, out);
     return cudaGetLastError();
 }
 
@@ -3505,7 +3534,7 @@ cudaError_t launch_half(size_t n, const LevelArrays<double> &a, const LevelArray
                         const LevelArrays<double> &out, cudaStream_t s)
 {
     note_launch();
-    k_half<<<red_grid(n), kRedThreads, 0, s>>>(n, a, b, out);
+    k_half<<<vec_grid(n), kRedThreads, 0, s>>>(n, a, b, out);
     return cudaGetLastError();
 }
 
@@ -3521,7 +3550,7 @@ cudaError_t launch_area_coeffs(size_t n, const LevelArrays<double> &area, const 
                                const LevelArrays<double> &out, cudaStream_t s)
 {
     note_launch();
-    k_area_coeffs<<<red_grid(n), kRedThreads, 0, s>>>(n, area, beta, out);
+    k_area_coeffs<<<vec_grid(n), kRedThreads, 0, s>>>(n, area, beta, out);
     return cudaGetLastError();
 }
 
@@ -3598,7 +3627,7 @@ template <typename Z>
 cudaError_t launch_pcg_dots(size_t n, const double *r, const Z *z, const Z *zo, double *partials, double *dscal,
                             int sz_slot, int so_slot, cudaStream_t s)
 {
-    const unsigned g = red_grid(n);
+    const unsigned g = vec_grid(n);
     note_launch();
     k_pcg_dots<Z><<<g, kRedThreads, 0, s>>>((unsigned)n, r, z, zo, dscal, sz_slot, so_slot, partials);
     return cudaGetLastError();
@@ -3623,7 +3652,7 @@ cudaError_t launch_pcg_dir(size_t n, const Z *z, double *d, double *dscal, int s
     if (sp.half && sizeof(Z) != 4) return cudaErrorInvalidValue;  // FP64 fields are never split
     if (so_slot >= 0 && sz_slot < 0) return cudaErrorInvalidValue;
     note_launch();
-    k_pcg_dir<Z><<<red_grid(n), kRedThreads, 0, s>>>((unsigned)n, z, d, dscal, sz_slot, so_slot, first, sp, partials);
+    k_pcg_dir<Z><<<sizeof(Z) == 8 ? vec_grid(n) : red_grid(n), kRedThreads, 0, s>>>((unsigned)n, z, d, dscal, sz_slot, so_slot, first, sp, partials);
     return cudaGetLastError();
 }
 template cudaError_t launch_pcg_dir<double>(size_t, const double *, double *, double *, int, int, int, cudaStream_t,
