@@ -687,11 +687,15 @@ __global__ void k_smooth_split(int nx, int ny, int nz, float h2, LevelArrays<flo
 // face arrays: a cell's low faces are the own colour's slots, its high faces the low faces of its
 // +x, +y and +z neighbours, i.e. the other colour's slots of its x-neighbour (as for p), mb + hx
 // and mb + hxy; six float4 and one scalar, each value used.
-template <int OFF, bool BAND, bool ZERO>
+// ROWS: 1 where a warp lies in one row (OFF_ is then the row's offset), 0 where it may hold several
+// rows of both parities (off: this thread's; selected per value, so that the warp does not run the
+// two parities one after the other).
+template <int ROWS, int OFF_, bool BAND, bool ZERO>
 __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, const LevelArrays<float> &S,
                                             const float *__restrict__ b, float *__restrict__ p, int colour, float4 rv,
-                                            int g, int j, int k)
+                                            int g, int j, int k, int off)
 {
+    const int OFF = ROWS ? OFF_ : off;
     const float v = rv.x;
     const int G = nx / 8;
     const size_t sxy = (size_t)nx * ny, half = sxy * nz / 2, hx = nx / 2, hxy = sxy / 2;
@@ -728,7 +732,9 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
     // b of this colour is read next a sweep later: loaded evict-first, so that it leaves L2 to the
     // iterate the next pass reads
     const float4 bv = __ldcs(reinterpret_cast<const float4 *>(bo + mb));
-    const float xs[6] = {OFF ? 0.f : oxe, ox.x, ox.y, ox.z, ox.w, OFF ? oxe : 0.f};  // slots mb-1 .. mb+4
+    // the x-neighbours of the four cells: slots mb-1+OFF .. mb+2+OFF and mb+OFF .. mb+3+OFF
+    const float xm[4] = {OFF ? ox.x : oxe, OFF ? ox.y : ox.x, OFF ? ox.z : ox.y, OFF ? ox.w : ox.z};
+    const float xp[4] = {xm[1], xm[2], xm[3], OFF ? oxe : ox.w};
     const float oy0[4] = {oym.x, oym.y, oym.z, oym.w}, oy1[4] = {oyp.x, oyp.y, oyp.z, oyp.w};
     const float oz0[4] = {ozm.x, ozm.y, ozm.z, ozm.w}, oz1[4] = {ozp.x, ozp.y, ozp.z, ozp.w};
     const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
@@ -750,7 +756,7 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
 #pragma unroll
         for (int t = 0; t < 4; t++) {
             const int i = 8 * g + 2 * t + OFF;
-            const float pxm = xs[t + OFF], pxp = xs[t + 1 + OFF];  // slots mb+t-1+OFF, mb+t+OFF
+            const float pxm = xm[t], pxp = xp[t];
             float s = 0.f;
             if (i > 0) s = fmaf(vx, pxm, s);
             if (i < nx - 1) s = fmaf(vx, pxp, s);
@@ -769,16 +775,17 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
         const float xe = (OFF && g < G - 1) ? S.bx[sn + mb + 4] : 0.f;
         const float4 yh = (j < ny - 1) ? *reinterpret_cast<const float4 *>(S.by + sn + mb + hx) : zero4;
         const float4 zh = (k < nz - 1) ? *reinterpret_cast<const float4 *>(S.bz + sn + mb + hxy) : zero4;
-        const float fxl[4] = {xl.x, xl.y, xl.z, xl.w}, fxh[5] = {xh.x, xh.y, xh.z, xh.w, xe};
+        // high x-faces: the other colour's slots mb+OFF .. mb+3+OFF, the x-neighbours' low faces
+        const float fxl[4] = {xl.x, xl.y, xl.z, xl.w};
+        const float fxh[4] = {OFF ? xh.y : xh.x, OFF ? xh.z : xh.y, OFF ? xh.w : xh.z, OFF ? xe : xh.w};
         const float fyl[4] = {yl.x, yl.y, yl.z, yl.w}, fyh[4] = {yh.x, yh.y, yh.z, yh.w};
         const float fzl[4] = {zl.x, zl.y, zl.z, zl.w}, fzh[4] = {zh.x, zh.y, zh.z, zh.w};
 #pragma unroll
         for (int t = 0; t < 4; t++) {
             const int i = 8 * g + 2 * t + OFF;
-            // high x-face: the other colour's slot mb+t+OFF, the x-neighbour's low face
-            const float bxl = fxl[t], bxh = i < nx - 1 ? fxh[t + OFF] : 0.f;
+            const float bxl = fxl[t], bxh = i < nx - 1 ? fxh[t] : 0.f;
             const float byl = fyl[t], byh = fyh[t], bzl = fzl[t], bzh = fzh[t];
-            const float pxm = xs[t + OFF], pxp = xs[t + 1 + OFF];
+            const float pxm = xm[t], pxp = xp[t];
             float s = 0.f;
             if (i > 0) s = fmaf(bxl, pxm, s);
             if (i < nx - 1) s = fmaf(bxh, pxp, s);
@@ -791,14 +798,14 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
     }
     *reinterpret_cast<float4 *>(own + mb) = make_float4(out[0], out[1], out[2], out[3]);
 }
-template <bool BAND, bool ZERO>
+template <bool BAND, bool ZERO, int ROWS>
 __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<float> S, const float *__restrict__ b,
                                 float *__restrict__ p, int colour, const float *__restrict__ urow,
                                 const float4 *__restrict__ arow, int rev)
 {
     // rev: the blocks take the planes (and rows) in descending order, so that a pass that follows
     // an ascending one starts on the data that pass touched last (still in L2)
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;  // (blockDim.x = 32 where ROWS = 1)
     const int by = rev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y;
     // the planes of the four quarters interleaved in the block order (0, nz/4, nz/2, 3nz/4, 1, ...):
     // the rows without a record gather in a band of planes (an interface), and interleaving runs
@@ -815,8 +822,10 @@ __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<fl
         const float v = urow ? urow[(size_t)k * ny + j] : 0.f;
         rv = make_float4(v, v, v, v);
     }
-    if ((j + k + colour) & 1) split4_body<1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k);
-    else split4_body<0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k);
+    const int off = (j + k + colour) & 1;
+    if (!ROWS) split4_body<0, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, off);
+    else if (off) split4_body<1, 1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 1);
+    else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 0);
 }
 
 // r = b - h^-2 sum_f beta_f (p_nb - p_c) at one fine cell (sum order x-,x+,y-,y+,z-,z+).
@@ -2991,6 +3000,22 @@ inline dim3 row_grid2(int threads_x, int ny, int nz)
     return dim3((unsigned)((threads_x + b.x - 1) / b.x), (unsigned)((ny + b.y - 1) / b.y), (unsigned)nz);
 }
 
+// Blocks of the finest FP32 level's kernels that take several cells along x per thread (rows of G threads):
+// 32 threads by 4 rows where G is a multiple of 32, else G cut into equal parts of at most 32 threads
+// by as many rows as make up to 128 threads, so that short rows do not leave lanes idle (at nx = 128 a
+// colour pass had 16 threads per row and ran half of each warp: 18.4 us per sweep, 15.6 us so; 192x160x224
+// 33.0 -> 30.4 us, 320x192x128 43.2 -> 37.2 us).  Rows of 32 threads keep the colour pass's body per row
+// parity: with the parity selected per value it took 63.5 us per sweep at 256^3 instead of 57.8.
+inline dim3 pair_block(int G)
+{
+    const int parts = (G + 31) / 32, x = (G + parts - 1) / parts;
+    return dim3((unsigned)x, (unsigned)(128 / x));
+}
+inline dim3 pair_grid(int G, int rows, int planes, dim3 block)
+{
+    return dim3((unsigned)((G + block.x - 1) / block.x), (unsigned)((rows + block.y - 1) / block.y), (unsigned)planes);
+}
+
 // Blocks of the grid-stride reductions: at most five per SM, so that the grid is one wave (the operator
 // of the CG holds six blocks per SM by its registers) and its end reads few partials, and on small
 // grids at least four cells per thread beyond two blocks per SM.  CG operator + update + dots and
@@ -3089,23 +3114,23 @@ cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, c
                                 const LevelArrays<float> *S)
 {
     note_launch();
-    if (d.nx % 8 == 0) {  // four cells per thread, blocks of 32 threads x 4 rows
+    if (d.nx % 8 == 0) {  // four cells per thread
         if (!S || !S->bx || !S->by || !S->bz) return cudaErrorInvalidValue;
-        const int G = d.nx / 8;
-        const dim3 grid((G + 31) / 32, (d.ny + 3) / 4, d.nz), block(32, 4);
+        const dim3 block = pair_block(d.nx / 8), grid = pair_grid(d.nx / 8, d.ny, d.nz, block);
+        auto go = [&](auto band, auto zer, auto rows) {
+            k_smooth_split4<decltype(band)::value, decltype(zer)::value, decltype(rows)::value ? 1 : 0>
+                <<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, rev);
+        };
+        auto go_rows = [&](auto band, auto zer) {
+            if (block.x == 32) go(band, zer, BoolTag<true>{});
+            else go(band, zer, BoolTag<false>{});
+        };
         if (arow) {
-            if (zero)
-                k_smooth_split4<true, true><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, rev);
-            else
-                k_smooth_split4<true, false><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow,
-                                                                    rev);
+            if (zero) go_rows(BoolTag<true>{}, BoolTag<true>{});
+            else go_rows(BoolTag<true>{}, BoolTag<false>{});
         } else {
-            if (zero)
-                k_smooth_split4<false, true><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow,
-                                                                    nullptr, rev);
-            else
-                k_smooth_split4<false, false><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow,
-                                                                     nullptr, rev);
+            if (zero) go_rows(BoolTag<false>{}, BoolTag<true>{});
+            else go_rows(BoolTag<false>{}, BoolTag<false>{});
         }
     } else {
         k_smooth_split<<<row_grid(d.nx / 2, d.ny, d.nz), kRowThreads, 0, s>>>(d.nx, d.ny, d.nz, h2, L, b, p, colour,
@@ -3136,7 +3161,7 @@ cudaError_t launch_restrict(Dims f, T ih2, const LevelArrays<T> &L, const T *b, 
     if constexpr (std::is_same<T, float>::value) {
         if (sp.half && f.nx % 8 == 0) {
             if (!S || !S->bx || !urow) return cudaErrorInvalidValue;
-            const dim3 g4((f.nx / 4 + 31) / 32, (f.ny / 2 + 3) / 4, f.nz / 2), b4(32, 4);
+            const dim3 b4 = pair_block(f.nx / 4), g4 = pair_grid(f.nx / 4, f.ny / 2, f.nz / 2, b4);
             if (arow)
                 k_restrict4<true><<<g4, b4, 0, s>>>(f.nx, f.ny, f.nz, ih2, *S, b, p, bc, urow, arow, rev);
             else
@@ -3172,7 +3197,7 @@ cudaError_t launch_prolong_red(Dims f, const T *ec, const T *dinv, T *p, cudaStr
     if constexpr (std::is_same<T, float>::value) {
         if (sp.half && f.nx % 8 == 0) {
             if (!urow) return cudaErrorInvalidValue;
-            const dim3 g4((f.nx / 4 + 31) / 32, (f.ny / 2 + 3) / 4, f.nz / 2), b4(32, 4);
+            const dim3 b4 = pair_block(f.nx / 4), g4 = pair_grid(f.nx / 4, f.ny / 2, f.nz / 2, b4);
             k_prolong_red4<<<g4, b4, 0, s>>>(f.nx, f.ny, f.nz, ec, dinv, p, arow ? &arow->x : urow, arow ? 4 : 1);
             return cudaGetLastError();
         }

@@ -94,3 +94,20 @@ def test_tail_slabs_identical_to_launches(mgp, shape, nu):
                 ctx.vcycle(rhs, p)
             out.append(p)
         assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1]), prec
+
+
+@pytest.mark.parametrize("shape", [(264, 16, 16), (320, 24, 16), (72, 24, 40), (256, 8, 16), (8, 16, 16)])
+def test_row_blocks_identical_to_natural_layout(mgp, shape):
+    """The finest colour passes, restriction and prolongation with rows that do and do not fill their
+    blocks' rows of 32 threads: bit for bit the cycle on the natural layout (fused sweeps)."""
+    case = synth.small_case(*shape, solid="ellipsoid", seed=53)
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    rhs = dev(case.rhs)
+    out = []
+    for sm in (1, 2):
+        ctx = mgp.Context(beta, case.h, prec="mixed", smoother=sm, coarse_max_cells=2048)
+        p = torch.zeros_like(rhs)
+        for _ in range(2):
+            ctx.vcycle(rhs, p)
+        out.append(p)
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
