@@ -97,6 +97,7 @@ struct mg_ctx {
     LevelArrays<double> rk_b1, rk_b2, rk_ut, rk_us, rk_r;
     double *rk_phis = nullptr;
     double *rk_work = nullptr;  // the momentum terms' per-cell fluxes and stresses
+    double *rec64 = nullptr;  // row records of the finest level's FP64 sweeps (MG_FP64, colour passes)
     float *urow0 = nullptr;  // uniform-row values of the finest FP32 level (with split0)
     // banded-row records of the finest FP32 level (with split0 and nx % 8 == 0), the two row
     // counts of the last hierarchy build, and whether its sweeps use the records (more banded
@@ -439,6 +440,7 @@ int tail_layout(const mg_ctx *c, const std::vector<LevelArrays<T>> &L, int ctas,
             v.P = (d.nz + ctas - 1) / ctas;
             v.h2 = (T)(c->hs[l + q] * c->hs[l + q]);
             v.ih2 = (T)(1.0 / (c->hs[l + q] * c->hs[l + q]));
+            v.sh2 = mg::scale2((double)v.h2);
             v.L = L[l + q];
             v.fnx = mg::make_fastdiv((unsigned)d.nx);
             v.fhx = mg::make_fastdiv((unsigned)std::max(d.nx / 2, 1));
@@ -501,6 +503,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     const mg::Split sp = (sizeof(T) == 4 && l == 0) ? c->split0 : mg::Split{};
     const float *urow = (sizeof(T) == 4 && l == 0) ? c->urow0 : nullptr;
     const float4 *arow = (sizeof(T) == 4 && l == 0 && c->banded) ? c->arow0 : nullptr;
+    const double *rec = (sizeof(T) == 8 && l == 0) ? c->rec64 : nullptr;
     T *cur = p, *alt = palt_of<T>(c, l);
     // plane order of the finest colour passes (pass_order = 1): each group of passes alternates
     // descending, ascending, ... so that every pass starts on the planes its predecessor (or the
@@ -531,8 +534,8 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
                 npass += skip ? 1 : 2;
             }
         } else {
-            if (!skip) CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first, s, 0, -1, zpass));
-            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first ^ 1, s));
+            if (!skip) CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first, s, zpass, rec));
+            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first ^ 1, s, false, rec));
         }
         zpass = false;
         skip = false;
@@ -829,6 +832,7 @@ int compute_hierarchy(mg_ctx *c, const double *const face_coeffs[3])
         CK(cudaMemcpyAsync(hcb + (size_t)a * nc, src[a], nc * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(c->hscal, c->dscal, mg::S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaEventRecord(c->ev_h, s));
+    if (c->rec64) CK(mg::launch_row_records64(c->dims[0], c->L64[0], c->rec64, s));
     if (c->o.prec == MG_MIXED) {
         // narrowed faces and 1/sum of them (the value the FP32 smoothers form on the fly); the
         // finest level's faces also in the colour-split layout
@@ -1146,6 +1150,10 @@ int mg_setup(mg_ctx **out, const mg_grid *g, const double *const face_coeffs[3],
         cudaEventCreateWithFlags(&c->ev_h, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(MG_ERR_CUDA, "mg_setup: pinned buffer / event creation failed"));
+    }
+    if (c->o.prec == MG_FP64 && c->o.smoother <= 1 && c->nlev >= 2) {
+        st = c->alloc(&c->rec64, 8 * (size_t)c->dims[0].ny * c->dims[0].nz);
+        if (st != MG_OK) return bail(st);
     }
     if (c->o.prec == MG_MIXED) {
         c->L32.resize(c->nlev);

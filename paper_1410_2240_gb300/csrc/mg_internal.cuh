@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -78,6 +79,19 @@ inline FastDiv make_fastdiv(unsigned d)
     return FastDiv{(unsigned)m, l < 1 ? l : 1u, l > 1 ? l - 1 : 0u};
 }
 
+// A factor f with the exponent e of f = 2^e where it is a power of two (ok), for products on the integer
+// pipe (mul_s2 in mg_kernels.cu)
+struct Scale2 {
+    double f;
+    int e, ok;
+};
+inline Scale2 scale2(double f)
+{
+    int ex;
+    const bool ok = std::frexp(f, &ex) == 0.5;
+    return Scale2{f, ex - 1, ok ? 1 : 0};
+}
+
 // Layout of the finest level's FP32 iterate and right-hand side.  half == 0: natural C order.
 // half == n / 2 (all dims even): colour-split, the cells of colour (i + j + k) & 1 == 0 in
 // [0, half) and of colour 1 in [half, n), cell c at slot c >> 1 of its colour's half.  Face
@@ -107,6 +121,7 @@ struct TailLevel {
     int P;                               // planes per CTA
     unsigned op, ob, ox, oy, oz, od;     // offsets in a CTA's memory (elements): p, b, faces, inverse diagonal
     T h2, ih2;
+    Scale2 sh2;                          // h2 as a factor
     LevelArrays<T> L;
     FastDiv fnx, fhx, fny, fP;           // division by nx, nx / 2, ny, P
 };
@@ -135,11 +150,16 @@ cudaError_t launch_restrict_coeffs(Dims fine, const double *bx, const double *by
 cudaError_t launch_level_f32(Dims d, const LevelArrays<double> &L, LevelArrays<float> &out, cudaStream_t s,
                              LevelArrays<float> *sf = nullptr, Split sp = {});
 
-// one colour of a red-black sweep on planes [z0, z1) (z1 < 0: to the last plane); zero: the
-// iterate is zero and is not read (the first pass of a cycle from a zero guess)
+// one colour of a red-black sweep; zero: the iterate is zero and is not read (the first pass of a
+// cycle from a zero guess)
+// rec (FP64, optional): the level's row records (launch_row_records64)
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          int z0 = 0, int z1 = -1, bool zero = false);
+                          bool zero = false, const double *rec = nullptr);
+// rec[8 r ..]: {vx, vy, vzl, vzh, 1 / (2 vx + 2 vy + vzl + vzh), 1 / (vx + 2 vy + vzl + vzh), 0, 0} for an interior
+// row r = k ny + j whose x-faces (walls aside), y-faces, low and high z-faces hold one positive value
+// each, zeros for any other; the inverses are the diagonal's (k_diag_inv) inside and at the x-walls
+cudaError_t launch_row_records64(Dims d, const LevelArrays<double> &L, double *rec, cudaStream_t s);
 // one colour of a red-black sweep on the colour-split layout (FP32, all dims even); urow (optional):
 // the level's uniform-row values, arow (optional, nx % 8 == 0, replaces urow in the sweep): its
 // banded-row records (launch_uniform_rows); rev: blocks take the planes in descending order; S

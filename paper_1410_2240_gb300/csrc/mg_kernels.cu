@@ -227,7 +227,11 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // clear sign bit; the coefficients, inverse diagonals and live masks it is applied to are never
 // NaN for finite input.  zero_bits(x) equals x == 0 for every x.
 __device__ __forceinline__ bool pos_bits(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
+// (from its two words: of the 64-bit pattern shifted left the compiler makes an FP64 comparison again)
+__device__ __forceinline__ bool zero_bits(double x)
+{
+    return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
+}
 __device__ __forceinline__ bool zero_bits(float x) { return (__float_as_int(x) << 1) == 0; }
 
 // ---------------------------------------------------------------------------
@@ -321,11 +325,7 @@ __device__ __forceinline__ double mul_pow2(double x, double f, int e)
 #endif
     return y;
 }
-// a power-of-two factor (ok: f = 2^e) or any other (ok = 0: a multiply)
-struct Scale2 {
-    double f;
-    int e, ok;
-};
+// the product with a power-of-two factor (ok: f = 2^e) or any other (ok = 0: a multiply)
 __device__ __forceinline__ double mul_s2(double x, const Scale2 &s) { return s.ok ? mul_pow2(x, s.f, s.e) : dmul_call(x, s.f); }
 
 // cell c = (i, j, k) and the neighbours its guards admit (i > 0: c - 1, i < nx - 1: c + 1, ...)
@@ -518,43 +518,129 @@ __device__ __forceinline__ T inv_diag(T stored, T bxl, T bxh, T byl, T byh, T bz
 // ---------------------------------------------------------------------------
 // Red-black Gauss-Seidel, one colour ((i+j+k) mod 2 == colour).  Each thread
 // owns the one cell of that colour in an x-pair of a row:
-//     p_c = dinv_c * (sum_f beta_f p_nb - h^2 b_c),  sum order x-,x+,y-,y+,z-,z+,
-// products accumulated with fused multiply-adds in that order.
+//     p_c = dinv_c * (sum_f beta_f p_nb - h^2 b_c),  faces x-,x+,y-,y+,z-,z+,
+// products accumulated with fused multiply-adds in that order; in FP32 from 0 with the right-hand
+// side last, in FP64 from -h^2 b_c: h^2 b is an exponent shift on the integer pipe where h is a power of
+// two, so an update is 7 FP64 operations instead of 8 (the pass is bound by them).
 // ---------------------------------------------------------------------------
-// one cell's update (shared by k_smooth and the coarse tail, so both round alike).  STORED: take
-// 1/sum from L.dinv also in FP32, where the hierarchy stores exactly inv_diag's value.  ZERO: the
-// iterate is zero (the first pass of a cycle from a zero guess): the neighbours are not read, the
-// products with +0 give the +0 sum the loads of a zeroed array would
-template <typename T, bool STORED = false, bool ZERO = false>
-__device__ __forceinline__ void smooth_cell(int i, int j, int k, int nx, int ny, int nz, T h2, const LevelArrays<T> &L,
-                                            const T *b, T *p)
+// the right-hand side's factor: h^2, and as a Scale2 (FP64)
+template <typename T>
+struct GsScale {
+    T h2;
+    Scale2 s;
+};
+template <typename T>
+GsScale<T> gs_scale(T h2)
 {
-    const size_t sxy = (size_t)nx * ny;
-    const size_t c = (size_t)k * sxy + (size_t)j * nx + i;
-    T s = T(0);
-    const T bxl = L.bx[c], bxh = (i < nx - 1) ? L.bx[c + 1] : T(0);
-    const T byl = L.by[c], byh = (j < ny - 1) ? L.by[c + nx] : T(0);
-    const T bzl = L.bz[c], bzh = (k < nz - 1) ? L.bz[c + sxy] : T(0);
-    auto nb = [&](size_t q) { return ZERO ? T(0) : p[q]; };
-    if (i > 0) s = fma(bxl, nb(c - 1), s);
-    if (i < nx - 1) s = fma(bxh, nb(c + 1), s);
-    if (j > 0) s = fma(byl, nb(c - nx), s);
-    if (j < ny - 1) s = fma(byh, nb(c + nx), s);
-    if (k > 0) s = fma(bzl, nb(c - sxy), s);
-    if (k < nz - 1) s = fma(bzh, nb(c + sxy), s);
-    const T d = (STORED || sizeof(T) == 8) ? L.dinv[c] : inv_diag<T>(T(0), bxl, bxh, byl, byh, bzl, bzh);
-    p[c] = d * fma(-h2, b[c], s);
+    return GsScale<T>{h2, scale2((double)h2)};
 }
+// what the products are added to, a product added, and the update from the sum.  The FP64 sum is kept with
+// its sign turned round, h^2 b - sum beta p (the same roundings): a negation of its own would be an FP64
+// addition, those of a product's factors are free.
+__device__ __forceinline__ double gs_start(double b, const GsScale<double> &g) { return mul_s2(b, g.s); }
+__device__ __forceinline__ float gs_start(float, const GsScale<float> &) { return 0.f; }
+__device__ __forceinline__ double gs_add(double beta, double p, double s) { return fma(beta, -p, s); }
+__device__ __forceinline__ float gs_add(float beta, float p, float s) { return fmaf(beta, p, s); }
+__device__ __forceinline__ double gs_update(double s, double, double d, const GsScale<double> &) { return -d * s; }
+__device__ __forceinline__ float gs_update(float s, float b, float d, const GsScale<float> &g) { return d * fmaf(-g.h2, b, s); }
 
-template <typename T, bool ZERO>
-__global__ void k_smooth(int nx, int ny, int nz, T h2, LevelArrays<T> L, const T *__restrict__ b,
-                         T *__restrict__ p, int colour, int z0)
+// ZERO: the iterate is zero (the first pass of a cycle from a zero guess): the products with it are
+// zeros, so only b and the inverse diagonal are read.  Both precisions take 1/sum from dinv (in FP32 the
+// hierarchy stores exactly inv_diag's value).  ROWS (FP64 finest level): rows with a record
+// (launch_row_records64) take the faces and the inverse diagonal from it, the same values: 24 bytes per
+// cell and pass instead of 56, since a pass that loads the faces is bound by HBM (0.139 ms at 256^3) as
+// much as by the FP64 unit (0.132 ms at 8 operations, 0.115 at 7).  Sweep at 256^3, FP64: 0.271 ms with
+// 8 operations and every face loaded, 0.257 with 7 and the short zero pass, 0.231 with the records
+// too (the average over the passes of a cycle from zero); 128^3 40.6 -> 34.2 us.
+template <typename T, bool ZERO, bool ROWS>
+__global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L, const T *__restrict__ b,
+                         T *__restrict__ p, int colour, const double2 *__restrict__ rec)
 {
-    const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z + z0;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
     const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((j + k + colour) & 1);
     if (i >= nx || j >= ny) return;
-    if (!ck_cell(((long long)k * ny + j) * nx + i, i, j, k, nx, ny, nz, CK_SMOOTH)) return;
-    smooth_cell<T, true, ZERO>(i, j, k, nx, ny, nz, h2, L, b, p);
+    const size_t sxy = (size_t)nx * ny;
+    const size_t c = (size_t)k * sxy + (size_t)j * nx + i;
+    if (!ck_cell((long long)c, i, j, k, nx, ny, nz, CK_SMOOTH)) return;
+    const T bc = b[c];
+    if (ZERO) {
+        p[c] = gs_update(gs_start(bc, gs), bc, L.dinv[c], gs);
+        return;
+    }
+    const bool xl = i > 0, xh = i < nx - 1, yl = j > 0, yh = j < ny - 1, zl = k > 0, zh = k < nz - 1;
+    // the neighbours are loaded before the row's record is known, so a row with one waits for one round trip
+    const T pxl = xl ? p[c - 1] : T(0), pxh = xh ? p[c + 1] : T(0);
+    const T pyl = yl ? p[c - nx] : T(0), pyh = yh ? p[c + nx] : T(0);
+    const T pzl = zl ? p[c - sxy] : T(0), pzh = zh ? p[c + sxy] : T(0);
+    T bxl, bxh, byl, byh, bzl, bzh, d;
+    bool loaded = false;
+    if constexpr (ROWS && sizeof(T) == 8) {
+        const double2 *r = rec + 4 * ((size_t)k * ny + j);
+        const double2 v0 = r[0];
+        if (!zero_bits(v0.x)) {
+            const double2 v1 = r[1];
+            bxl = bxh = v0.x;
+            byl = byh = v0.y;
+            bzl = v1.x;
+            bzh = v1.y;
+            // an address, not a branch: lanes apart at a wall would run the update's last product twice
+            d = reinterpret_cast<const double *>(r)[xl && xh ? 4 : 5];
+            loaded = true;
+        }
+    }
+    if (!loaded) {
+        bxl = L.bx[c];
+        bxh = xh ? L.bx[c + 1] : T(0);
+        byl = L.by[c];
+        byh = yh ? L.by[c + nx] : T(0);
+        bzl = L.bz[c];
+        bzh = zh ? L.bz[c + sxy] : T(0);
+        d = L.dinv[c];
+    }
+    T s = gs_start(bc, gs);
+    if (xl) s = gs_add(bxl, pxl, s);
+    if (xh) s = gs_add(bxh, pxh, s);
+    if (yl) s = gs_add(byl, pyl, s);
+    if (yh) s = gs_add(byh, pyh, s);
+    if (zl) s = gs_add(bzl, pzl, s);
+    if (zh) s = gs_add(bzh, pzh, s);
+    p[c] = gs_update(s, bc, d, gs);
+}
+
+// the row records of an FP64 level, one warp per row (as k_uniform_rows)
+__global__ void k_row_records64(int nx, int ny, int nz, const double *__restrict__ bx, const double *__restrict__ by,
+                                const double *__restrict__ bz, double2 *__restrict__ rec)
+{
+    const int lane = threadIdx.x & 31, r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r >= ny * nz) return;
+    const int j = r % ny, k = r / ny;
+    const size_t sxy = (size_t)nx * ny, c0 = (size_t)r * nx;
+    const bool inner = nx > 1 && j > 0 && k > 0 && j < ny - 1 && k < nz - 1;
+    double vx = 0.0, vy = 0.0, vzl = 0.0, vzh = 0.0;
+    if (inner) {
+        vx = bx[c0 + 1];
+        vy = by[c0];
+        vzl = bz[c0];
+        vzh = bz[c0 + sxy];
+    }
+    bool ok = inner && pos_bits(vx) && pos_bits(vy) && pos_bits(vzl) && pos_bits(vzh);
+    if (ok)  // warp-uniform
+        for (int i = lane; i < nx; i += 32) {
+            const size_t c = c0 + i;
+            const bool cell = (i == 0 || same_bits(bx[c], vx)) & same_bits(by[c], vy) & same_bits(by[c + nx], vy) &
+                              same_bits(bz[c], vzl) & same_bits(bz[c + sxy], vzh);
+            ok = ok & cell;
+        }
+    ok = __all_sync(0xffffffffu, ok);
+    if (lane != 0) return;
+    double i6 = 0.0, i5 = 0.0;
+    if (ok) {
+        i6 = div_call(1.0, ((((vx + vx) + vy) + vy) + vzl) + vzh);
+        i5 = div_call(1.0, (((vx + vy) + vy) + vzl) + vzh);
+    }
+    rec[4 * (size_t)r] = ok ? make_double2(vx, vy) : make_double2(0.0, 0.0);
+    rec[4 * (size_t)r + 1] = ok ? make_double2(vzl, vzh) : make_double2(0.0, 0.0);
+    rec[4 * (size_t)r + 2] = make_double2(i6, i5);
 }
 
 // Colour-split layout (Split in mg_internal.cuh): slot of natural cell c in a row of parity
@@ -693,7 +779,7 @@ __global__ void k_smooth_split(int nx, int ny, int nz, float h2, LevelArrays<flo
 template <int ROWS, int OFF_, bool BAND, bool ZERO>
 __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, const LevelArrays<float> &S,
                                             const float *__restrict__ b, float *__restrict__ p, int colour, float4 rv,
-                                            int g, int j, int k, int off)
+                                            int g, int j, int k, int off, const float *__restrict__ dinv)
 {
     const int OFF = ROWS ? OFF_ : off;
     const float v = rv.x;
@@ -739,7 +825,14 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
     const float oz0[4] = {ozm.x, ozm.y, ozm.z, ozm.w}, oz1[4] = {ozp.x, ozp.y, ozp.z, ozp.w};
     const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
     float out[4];
-    if (v != 0.f) {
+    if (ZERO && v == 0.f) {
+        // the products are zeros: 1/sum as the hierarchy stores it (natural order: this colour's are every
+        // second value of the eight) instead of the six faces it is the inverse of
+        const float4 d0 = *reinterpret_cast<const float4 *>(dinv + 2 * mb), d1 = *reinterpret_cast<const float4 *>(dinv + 2 * mb + 4);
+        const float dd[4] = {OFF ? d0.y : d0.x, OFF ? d0.w : d0.z, OFF ? d1.y : d1.x, OFF ? d1.w : d1.z};
+#pragma unroll
+        for (int t = 0; t < 4; t++) out[t] = dd[t] * fmaf(-h2, bb[t], 0.f);
+    } else if (v != 0.f) {
         // a row with a record: the diagonal is 6v, or 5v at an x-wall (the sums of inv_diag, in its
         // order: 0 + v = v + 0 = v), so two divisions serve the thread's four cells; on a banded
         // row the same with vx, vy, vzl, vzh in their places
@@ -801,7 +894,7 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
 template <bool BAND, bool ZERO, int ROWS>
 __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<float> S, const float *__restrict__ b,
                                 float *__restrict__ p, int colour, const float *__restrict__ urow,
-                                const float4 *__restrict__ arow, int rev)
+                                const float4 *__restrict__ arow, int rev, const float *__restrict__ dinv)
 {
     // rev: the blocks take the planes (and rows) in descending order, so that a pass that follows
     // an ascending one starts on the data that pass touched last (still in L2)
@@ -823,9 +916,9 @@ __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<fl
         rv = make_float4(v, v, v, v);
     }
     const int off = (j + k + colour) & 1;
-    if (!ROWS) split4_body<0, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, off);
-    else if (off) split4_body<1, 1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 1);
-    else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 0);
+    if (!ROWS) split4_body<0, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, off, dinv);
+    else if (off) split4_body<1, 1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 1, dinv);
+    else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 0, dinv);
 }
 
 // r = b - h^-2 sum_f beta_f (p_nb - p_c) at one fine cell (sum order x-,x+,y-,y+,z-,z+).
@@ -1342,7 +1435,7 @@ __global__ void k_prolong_red4(int nx, int ny, int nz, const float *__restrict__
 // ---------------------------------------------------------------------------
 template <typename T, int TX, int TY>
 __global__ void __launch_bounds__((TX + 4) * (TY + 4))
-k_rb_sweep(int nx, int ny, int nz, int zc, T h2, LevelArrays<T> L, const T *__restrict__ b,
+k_rb_sweep(int nx, int ny, int nz, int zc, GsScale<T> gs, LevelArrays<T> L, const T *__restrict__ b,
            const T *__restrict__ p_old, T *__restrict__ p_new, int first)
 {
     constexpr int W = TX + 4, H = TY + 4;
@@ -1397,14 +1490,14 @@ k_rb_sweep(int nx, int ny, int nz, int zc, T h2, LevelArrays<T> L, const T *__re
         if (ring1 && s >= 0 && s < nz && ((i + j + s) & 1) == first) {
             const T bxh = xhi ? sbx[cur][ly][lx + 1] : T(0), byh = yhi ? sby[cur][ly + 1][lx] : T(0);
             const T bzh = (s < nz - 1) ? bz_p1 : T(0);
-            T acc = T(0);
-            if (xlo) acc = fma(bx_0, sp[cur][ly][lx - 1], acc);
-            if (xhi) acc = fma(bxh, sp[cur][ly][lx + 1], acc);
-            if (ylo) acc = fma(by_0, sp[cur][ly - 1][lx], acc);
-            if (yhi) acc = fma(byh, sp[cur][ly + 1][lx], acc);
-            if (s > 0) acc = fma(bz_0, q_m1, acc);
-            if (s < nz - 1) acc = fma(bz_p1, q_p1, acc);
-            q_0 = inv_diag<T>(di_0, bx_0, bxh, by_0, byh, bz_0, bzh) * fma(-h2, b_0, acc);
+            T acc = gs_start(b_0, gs);
+            if (xlo) acc = gs_add(bx_0, sp[cur][ly][lx - 1], acc);
+            if (xhi) acc = gs_add(bxh, sp[cur][ly][lx + 1], acc);
+            if (ylo) acc = gs_add(by_0, sp[cur][ly - 1][lx], acc);
+            if (yhi) acc = gs_add(byh, sp[cur][ly + 1][lx], acc);
+            if (s > 0) acc = gs_add(bz_0, q_m1, acc);
+            if (s < nz - 1) acc = gs_add(bz_p1, q_p1, acc);
+            q_0 = gs_update(acc, b_0, inv_diag<T>(di_0, bx_0, bxh, by_0, byh, bz_0, bzh), gs);
             sp[cur][ly][lx] = q_0;
         }
         __syncthreads();
@@ -1414,14 +1507,14 @@ k_rb_sweep(int nx, int ny, int nz, int zc, T h2, LevelArrays<T> L, const T *__re
             if (((i + j + z) & 1) == second) {
                 const T bxh = xhi ? sbx[prv][ly][lx + 1] : T(0), byh = yhi ? sby[prv][ly + 1][lx] : T(0);
                 const T bzh = (z < nz - 1) ? bz_0 : T(0);
-                T acc = T(0);
-                if (xlo) acc = fma(bx_m1, sp[prv][ly][lx - 1], acc);
-                if (xhi) acc = fma(bxh, sp[prv][ly][lx + 1], acc);
-                if (ylo) acc = fma(by_m1, sp[prv][ly - 1][lx], acc);
-                if (yhi) acc = fma(byh, sp[prv][ly + 1][lx], acc);
-                if (z > 0) acc = fma(bz_m1, q_m2, acc);
-                if (z < nz - 1) acc = fma(bz_0, q_0, acc);
-                q_m1 = inv_diag<T>(di_m1, bx_m1, bxh, by_m1, byh, bz_m1, bzh) * fma(-h2, b_m1, acc);
+                T acc = gs_start(b_m1, gs);
+                if (xlo) acc = gs_add(bx_m1, sp[prv][ly][lx - 1], acc);
+                if (xhi) acc = gs_add(bxh, sp[prv][ly][lx + 1], acc);
+                if (ylo) acc = gs_add(by_m1, sp[prv][ly - 1][lx], acc);
+                if (yhi) acc = gs_add(byh, sp[prv][ly + 1][lx], acc);
+                if (z > 0) acc = gs_add(bz_m1, q_m2, acc);
+                if (z < nz - 1) acc = gs_add(bz_0, q_0, acc);
+                q_m1 = gs_update(acc, b_m1, inv_diag<T>(di_m1, bx_m1, bxh, by_m1, byh, bz_m1, bzh), gs);
             }
             p_new[(size_t)z * sxy + col] = q_m1;
         }
@@ -1517,6 +1610,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
         const T *const above = rank + 1 < ncta ? cl.map_shared_rank(p, rank + 1) : p;
         T fxl[kTailCells][2], fxh[kTailCells][2], fyl[kTailCells][2], fyh[kTailCells][2], fzl[kTailCells][2],
             fzh[kTailCells][2], fd[kTailCells][2], fb[kTailCells][2];
+        const GsScale<T> gs{v.h2, v.sh2};
         const T *zl[kTailCells], *zh[kTailCells];  // the planes below and above (colour 0)
         unsigned odd[kTailCells];                   // (j + k) & 1
 #pragma unroll
@@ -1549,17 +1643,17 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
             for (int e = 0; e < kTailCells; e++) {
                 const unsigned t = tid + e * nthr;
                 if (t >= total) break;
-                T s = T(0);
+                T s = gs_start(fb[e][q], gs);
                 if (!zero) {
                     const T *const ot = p + o * H + t, *const ox = ot + (odd[e] ^ q);
-                    s = fma(fxl[e][q], ox[-1], s);
-                    s = fma(fxh[e][q], ox[0], s);
-                    s = fma(fyl[e][q], *(ot - hx), s);
-                    s = fma(fyh[e][q], *(ot + hx), s);
-                    s = fma(fzl[e][q], zl[e][o * H], s);
-                    s = fma(fzh[e][q], zh[e][o * H], s);
+                    s = gs_add(fxl[e][q], ox[-1], s);
+                    s = gs_add(fxh[e][q], ox[0], s);
+                    s = gs_add(fyl[e][q], *(ot - hx), s);
+                    s = gs_add(fyh[e][q], *(ot + hx), s);
+                    s = gs_add(fzl[e][q], zl[e][o * H], s);
+                    s = gs_add(fzh[e][q], zh[e][o * H], s);
                 }
-                p[q * H + t] = fd[e][q] * fma(-v.h2, fb[e][q], s);
+                p[q * H + t] = gs_update(s, fb[e][q], fd[e][q], gs);
             }
             zero = false;
             cl.sync();
@@ -2446,7 +2540,7 @@ __global__ void k_phi_grad(int nx, int ny, int nz, double neg_half_drho, const d
             double tx_hi = 0.0, ty_hi = 0.0;
             if (i < nx - 1) tx_hi = threadIdx.x < W - 1 ? buf[0][t + 1] : sq_mul_call(bx[c + 1], gbx[c + 1]);
             if (j < ny - 1) ty_hi = threadIdx.y < R - 1 ? buf[1][t + W] : sq_mul_call(by[c + nx], gby[c + nx]);
-            double s = (__double_as_longlong(tx) << 1) == 0 ? 0.0 : tx;  // 0 + tx
+            double s = zero_bits(tx) ? 0.0 : tx;  // 0 + tx
             if (i < nx - 1) s = __dadd_rn(s, tx_hi);
             s = __dadd_rn(s, ty);
             if (j < ny - 1) s = __dadd_rn(s, ty_hi);
@@ -2964,13 +3058,6 @@ __global__ void k_comp_center(unsigned n, const double *__restrict__ v, const in
     }
 }
 
-// f as a Scale2 (ok when f = 2^e)
-inline Scale2 scale2(double f)
-{
-    int ex;
-    const bool ok = std::frexp(f, &ex) == 0.5;
-    return Scale2{f, ex - 1, ok ? 1 : 0};
-}
 // 1/h as a Scale2 for div_h: ok when h is a power of two (h = 2^(ex-1), 1/h = 2^(1-ex) exactly)
 inline Scale2 inv_scale2(double h)
 {
@@ -3092,22 +3179,30 @@ cudaError_t launch_restrict_coeffs(Dims f, const double *bx, const double *by, c
 
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          int z0, int z1, bool zero)
+                          bool zero, const double *rec)
 {
-    if (z1 < 0) z1 = d.nz;
-    if (z1 <= z0) return cudaSuccess;
     note_launch();
-    const dim3 g = row_grid2((d.nx + 1) / 2, d.ny, z1 - z0), blk = row_block2((d.nx + 1) / 2);
-    if (zero)
-        k_smooth<T, true><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, h2, L, b, p, colour, z0);
-    else
-        k_smooth<T, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, h2, L, b, p, colour, z0);
+    const dim3 g = row_grid2((d.nx + 1) / 2, d.ny, d.nz), blk = row_block2((d.nx + 1) / 2);
+    const GsScale<T> gs = gs_scale<T>(h2);
+    const double2 *r2 = reinterpret_cast<const double2 *>(rec);
+    if (zero) k_smooth<T, true, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
+    else if (sizeof(T) == 8 && rec) k_smooth<T, false, sizeof(T) == 8><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, r2);
+    else k_smooth<T, false, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
     return cudaGetLastError();
 }
 template cudaError_t launch_smooth<double>(Dims, double, const LevelArrays<double> &, const double *, double *, int,
-                                           cudaStream_t, int, int, bool);
+                                           cudaStream_t, bool, const double *);
 template cudaError_t launch_smooth<float>(Dims, float, const LevelArrays<float> &, const float *, float *, int,
-                                          cudaStream_t, int, int, bool);
+                                          cudaStream_t, bool, const double *);
+
+cudaError_t launch_row_records64(Dims d, const LevelArrays<double> &L, double *rec, cudaStream_t s)
+{
+    const int rows = d.ny * d.nz, warps = 8;
+    note_launch();
+    k_row_records64<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(d.nx, d.ny, d.nz, L.bx, L.by, L.bz,
+                                                                       reinterpret_cast<double2 *>(rec));
+    return cudaGetLastError();
+}
 
 cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, int colour,
                                 cudaStream_t s, const float *urow, const float4 *arow, int rev, bool zero,
@@ -3119,7 +3214,7 @@ cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, c
         const dim3 block = pair_block(d.nx / 8), grid = pair_grid(d.nx / 8, d.ny, d.nz, block);
         auto go = [&](auto band, auto zer, auto rows) {
             k_smooth_split4<decltype(band)::value, decltype(zer)::value, decltype(rows)::value ? 1 : 0>
-                <<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, rev);
+                <<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, rev, L.dinv);
         };
         auto go_rows = [&](auto band, auto zer) {
             if (block.x == 32) go(band, zer, BoolTag<true>{});
@@ -3251,7 +3346,8 @@ cudaError_t launch_rb_sweep(Dims d, T h2, const LevelArrays<T> &L, const T *b, c
     if (zc > d.nz) zc = d.nz;
     const dim3 grid((unsigned)tx, (unsigned)ty, (unsigned)((d.nz + zc - 1) / zc));
     note_launch();
-    k_rb_sweep<T, TX, TY><<<grid, (TX + 4) * (TY + 4), 0, s>>>(d.nx, d.ny, d.nz, zc, h2, L, b, p_old, p_new, first);
+    k_rb_sweep<T, TX, TY><<<grid, (TX + 4) * (TY + 4), 0, s>>>(d.nx, d.ny, d.nz, zc, gs_scale<T>(h2), L, b, p_old, p_new,
+                                                              first);
     return cudaGetLastError();
 }
 template cudaError_t launch_rb_sweep<double>(Dims, double, const LevelArrays<double> &, const double *,

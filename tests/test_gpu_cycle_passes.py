@@ -96,7 +96,7 @@ def test_tail_slabs_identical_to_launches(mgp, shape, nu):
         assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1]), prec
 
 
-@pytest.mark.parametrize("shape", [(264, 16, 16), (320, 24, 16), (72, 24, 40), (256, 8, 16), (8, 16, 16)])
+@pytest.mark.parametrize("shape", [(264, 16, 16), (320, 24, 16), (72, 24, 40), (256, 16, 32), (8, 16, 16)])
 def test_row_blocks_identical_to_natural_layout(mgp, shape):
     """The finest colour passes, restriction and prolongation with rows that do and do not fill their
     blocks' rows of 32 threads: bit for bit the cycle on the natural layout (fused sweeps)."""
@@ -106,6 +106,32 @@ def test_row_blocks_identical_to_natural_layout(mgp, shape):
     out = []
     for sm in (1, 2):
         ctx = mgp.Context(beta, case.h, prec="mixed", smoother=sm, coarse_max_cells=2048)
+        p = torch.zeros_like(rhs)
+        for _ in range(2):
+            ctx.vcycle(rhs, p)
+        out.append(p)
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("shape,stretched", [((48, 16, 24), False), ((36, 32, 32), False), ((64, 32, 32), True),
+                                             ((10, 16, 16), True)])
+def test_fp64_row_records_identical_to_loaded_faces(mgp, shape, stretched):
+    """FP64 colour passes that take a row's faces and inverse diagonals from its record, uniform or
+    one value per kind of face (a grid stretched in z): bit for bit the fused sweeps, which load every
+    face."""
+    nx, ny, nz = shape
+    case = synth.small_case(nx, ny, nz, solid="ellipsoid", interface="flat", seed=54)
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    h, area = case.h, None
+    if stretched:
+        w = [dev(np.full(nx, h)), dev(np.full(ny, h)), dev(synth.stretched_widths(nz))]
+        beta, area = mgp.stretched_metrics(*w, beta)
+        h = 1.0
+    rhs = dev(case.rhs)
+    out = []
+    for sm in (1, 2):
+        ctx = mgp.Context(beta, h, smoother=sm, coarse_max_cells=2048)
+        ctx.set_face_areas(area)
         p = torch.zeros_like(rhs)
         for _ in range(2):
             ctx.vcycle(rhs, p)
