@@ -185,7 +185,7 @@ template <bool B>
 struct BoolTag {
     static constexpr bool value = B;
 };
-// Kernels that share face products along rows (k_phi_grad, k_divergence_mul): blocks of at most
+// Kernels that share values along rows (k_phi_grad, k_divergence_mul, k_mom_parts): blocks of at most
 // kPhiThreads threads over rows of at most kPhiW cells, kPhiRun planes per block.
 constexpr int kPhiW = 256, kPhiThreads = 512, kPhiRun = 8;
 
@@ -307,8 +307,8 @@ __device__ __noinline__ double sq_mul_call(double b, double g) { return __dmul_r
 
 // x * f for f = 2^e, bit for bit the product __dmul_rn(x, f), on the integer pipe where x and the
 // product are normal numbers: e added to the exponent field (the FP64 unit is the limiting
-// resource of the FP64 set-up and projection passes).  Zeros, subnormals, infinities, NaNs and
-// products outside the normal range take the multiply (a call).  The check build compares every
+// resource of the FP64 set-up and projection passes).  Zeros stay what they are (f > 0); subnormals,
+// infinities, NaNs and products outside the normal range take the multiply (a call).  The check build compares every
 // result with the multiply.
 __device__ __forceinline__ double mul_pow2(double x, double f, int e)
 {
@@ -317,6 +317,8 @@ __device__ __forceinline__ double mul_pow2(double x, double f, int e)
     double y;
     if ((unsigned)(ex - 1) < 2046u && (unsigned)(ex + e - 1) < 2046u)
         y = __hiloint2double(hi + e * (1 << 20), lo);
+    else if ((((unsigned)hi << 1) | (unsigned)lo) == 0u)
+        y = x;
     else
         y = dmul_call(x, f);
 #ifdef MGP_CHECK
@@ -326,6 +328,11 @@ __device__ __forceinline__ double mul_pow2(double x, double f, int e)
     return y;
 }
 // the product with a power-of-two factor (ok: f = 2^e) or any other (ok = 0: a multiply)
+// -x, exactly, on the integer pipe (a negation that no operand takes is an FP64 addition)
+__device__ __forceinline__ double neg_bits(double x)
+{
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+}
 __device__ __forceinline__ double mul_s2(double x, const Scale2 &s) { return s.ok ? mul_pow2(x, s.f, s.e) : dmul_call(x, s.f); }
 
 // cell c = (i, j, k) and the neighbours its guards admit (i > 0: c - 1, i < nx - 1: c + 1, ...)
@@ -2141,16 +2148,32 @@ __global__ void k_rk_combine(size_t n, LevelArrays<double> a, LevelArrays<double
 // open face's R from the values bracketing it.  A face's F_ab and S_ab are the same numbers
 // whichever of the four faces at the edge uses them (the product and the sum commute exactly), so
 // R is bitwise the per-face evaluation, with a third of its FP64 operations.
+//
+// Both passes are bound by the FP64 unit, so what is not an addition or a general product stays off it:
+// the halvings, doublings and quarterings, and the products with 1/h where h is a power of two (POW2), are exponent shifts
+// on the integer pipe; a cell's viscosity is formed once per block (shared memory) instead of by each of the
+// seven cells that use it; the terms a call leaves out (CONV, VISC) are not formed, their share of R
+// being a zero.  FP64 operations per cell: about 85 (106 where h is no power of two), 134 with all of that on the
+// FP64 unit.  At 256^3: 2.79 ms (4.23 ms), convective terms alone 1.03 ms, viscous alone 1.84 ms, gravity alone
+// 0.08 ms (4.23 ms each); 251x190x133 1.35 ms (1.64 ms).
 // ---------------------------------------------------------------------------
 struct MomArgs {
-    int nx, ny, nz, convect;
-    double ih, mu_air, dmu, inv_re, g;
+    int nx, ny, nz;
+    Scale2 ih;
+    double mu_air, dmu, inv_re, g;
     const double *phi;
     LevelArrays<double> beta, u, r;
     double *w;  // 12 arrays of n: C_x, C_y, C_z, T_x, T_y, T_z, F_xy, F_xz, F_yz, S_xy, S_xz, S_yz
 };
 
 __device__ __forceinline__ int clamp_idx(int v, int hi) { return v < 0 ? 0 : (v > hi ? hi : v); }
+
+// x / h as the product with 1/h
+template <bool POW2>
+__device__ __forceinline__ double mom_ih(const MomArgs &m, double x)
+{
+    return POW2 ? mul_pow2(x, m.ih.f, m.ih.e) : __dmul_rn(x, m.ih.f);
+}
 
 // velocity of axis AX on its face (i, j, k): 0 at the high wall of its own axis, the other two
 // indices mirrored into the domain
@@ -2165,6 +2188,7 @@ __device__ __forceinline__ double mom_vel(const MomArgs &m, int i, int j, int k)
     return u[((size_t)k * m.ny + j) * m.nx + i];
 }
 
+// viscosity of cell (i, j, k), the indices mirrored into the domain
 __device__ __forceinline__ double mom_mu(const MomArgs &m, int i, int j, int k)
 {
     i = clamp_idx(i, m.nx - 1);
@@ -2173,114 +2197,129 @@ __device__ __forceinline__ double mom_mu(const MomArgs &m, int i, int j, int k)
     return __dadd_rn(m.mu_air, __dmul_rn(m.dmu, m.phi[((size_t)k * m.ny + j) * m.nx + i]));
 }
 
-// centre flux and stress of axis A at cell (i, j, k) (mu: the cell's viscosity)
-template <int A>
-__device__ __forceinline__ void mom_centre(const MomArgs &m, int i, int j, int k, double mu, double &C, double &T)
+// centre flux and stress of axis A at cell (i, j, k) (mu: the cell's viscosity) into their arrays at c
+template <int A, bool CONV, bool VISC, bool POW2>
+__device__ __forceinline__ void mom_centre(const MomArgs &m, size_t n, size_t c, int i, int j, int k, double mu)
 {
     constexpr int ai = A == 0, aj = A == 1, ak = A == 2;
     const double u0 = mom_vel<A>(m, i, j, k), u1 = mom_vel<A>(m, i + ai, j + aj, k + ak);
-    const double U = __dmul_rn(0.5, __dadd_rn(u0, u1));
-    C = __dmul_rn(U, U);
-    T = __dmul_rn(__dmul_rn(2.0, mu), __dmul_rn(__dsub_rn(u1, u0), m.ih));
+    if (CONV) {
+        const double U = mul_pow2(__dadd_rn(u0, u1), 0.5, -1);
+        m.w[A * n + c] = __dmul_rn(U, U);
+    }
+    if (VISC) m.w[(3 + A) * n + c] = __dmul_rn(mul_pow2(mu, 2.0, 1), mom_ih<POW2>(m, __dsub_rn(u1, u0)));
 }
 
 // flux and shear of plane (A, B), A < B, at the low edge of cell (i, j, k); mc, ma, mb, mab: the
 // viscosities of the cell and of its neighbours below along A, along B, along both
-template <int A, int B>
-__device__ __forceinline__ void mom_edge(const MomArgs &m, int i, int j, int k, double mc, double ma, double mb,
-                                         double mab, double &F, double &S)
+template <int A, int B, bool CONV, bool VISC, bool POW2>
+__device__ __forceinline__ void mom_edge(const MomArgs &m, size_t n, size_t c, int i, int j, int k, double mc, double ma,
+                                         double mb, double mab)
 {
     constexpr int ai = A == 0, aj = A == 1, ak = A == 2, bi = B == 0, bj = B == 1, bk = B == 2;
+    constexpr int slot = A + B - 1;  // xy, xz, yz
     const double ua0 = mom_vel<A>(m, i - bi, j - bj, k - bk), ua1 = mom_vel<A>(m, i, j, k);
     const double ub0 = mom_vel<B>(m, i - ai, j - aj, k - ak), ub1 = mom_vel<B>(m, i, j, k);
-    F = __dmul_rn(__dmul_rn(0.5, __dadd_rn(ub0, ub1)), __dmul_rn(0.5, __dadd_rn(ua0, ua1)));
-    const double me = __dmul_rn(0.25, __dadd_rn(__dadd_rn(__dadd_rn(mab, mb), ma), mc));
-    S = __dmul_rn(me, __dadd_rn(__dmul_rn(__dsub_rn(ua1, ua0), m.ih), __dmul_rn(__dsub_rn(ub1, ub0), m.ih)));
+    if (CONV)
+        m.w[(6 + slot) * n + c] =
+            __dmul_rn(mul_pow2(__dadd_rn(ub0, ub1), 0.5, -1), mul_pow2(__dadd_rn(ua0, ua1), 0.5, -1));
+    if (VISC) {
+        const double me = mul_pow2(__dadd_rn(__dadd_rn(__dadd_rn(mab, mb), ma), mc), 0.25, -2);
+        m.w[(9 + slot) * n + c] =
+            __dmul_rn(me, __dadd_rn(mom_ih<POW2>(m, __dsub_rn(ua1, ua0)), mom_ih<POW2>(m, __dsub_rn(ub1, ub0))));
+    }
 }
 
+// blocks as k_phi_grad's (W x R threads, at most kPhiThreads, kPhiRun planes up z); the viscosities of a plane
+// of the block, with those of the row and the column before it, in one of three buffers by plane
+// (a buffer is written again three planes later: one barrier per plane)
+template <bool CONV, bool VISC, bool POW2>
 __global__ void k_mom_parts(MomArgs m)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
-    if (i >= m.nx || j >= m.ny) return;
-    const size_t n = (size_t)m.nx * m.ny * m.nz, c = ((size_t)k * m.ny + j) * m.nx + i;
-    if (!MG_CK(c, c, (long long)n, CK_MOMENTUM)) return;
-    const double mc = mom_mu(m, i, j, k), mx = mom_mu(m, i - 1, j, k), my = mom_mu(m, i, j - 1, k),
-                 mz = mom_mu(m, i, j, k - 1), mxy = mom_mu(m, i - 1, j - 1, k), mxz = mom_mu(m, i - 1, j, k - 1),
-                 myz = mom_mu(m, i, j - 1, k - 1);
-    double C, T, F, S;
-    mom_centre<0>(m, i, j, k, mc, C, T);
-    m.w[c] = C;
-    m.w[3 * n + c] = T;
-    mom_centre<1>(m, i, j, k, mc, C, T);
-    m.w[n + c] = C;
-    m.w[4 * n + c] = T;
-    mom_centre<2>(m, i, j, k, mc, C, T);
-    m.w[2 * n + c] = C;
-    m.w[5 * n + c] = T;
-    // in cell-index order: the cell below along both axes, below along the higher axis, below along
-    // the lower axis, the cell itself
-    mom_edge<0, 1>(m, i, j, k, mc, mx, my, mxy, F, S);
-    m.w[6 * n + c] = F;
-    m.w[9 * n + c] = S;
-    mom_edge<0, 2>(m, i, j, k, mc, mx, mz, mxz, F, S);
-    m.w[7 * n + c] = F;
-    m.w[10 * n + c] = S;
-    mom_edge<1, 2>(m, i, j, k, mc, my, mz, myz, F, S);
-    m.w[8 * n + c] = F;
-    m.w[11 * n + c] = S;
-}
-
-// edge value of plane (A, B) (either order) at the low edge of cell (i, j, k), which may lie on the
-// high wall of the other axis (one past the last cell): there the normal velocity of the wall and
-// the mirrored tangential velocity make both the flux and the shear zero
-template <int A, int B>
-__device__ __forceinline__ void mom_edge_at(const MomArgs &m, size_t n, int i, int j, int k, double &F, double &S)
-{
-    constexpr int lo = A < B ? A : B, hi = A < B ? B : A;
-    constexpr int slot = (lo == 0 && hi == 1) ? 0 : ((lo == 0) ? 1 : 2);
-    if (i >= m.nx || j >= m.ny || k >= m.nz) {
-        F = 0.0;
-        S = 0.0;
-        return;
+    __shared__ double sh[VISC ? 3 : 1][VISC ? kPhiThreads + kPhiW + 4 : 1];  // (R + 1) (W + 1): at most 3 x 257
+    const int W = blockDim.x, R = blockDim.y, tx = threadIdx.x, ty = threadIdx.y;
+    const int i = blockIdx.x * W + tx, j = blockIdx.y * R + ty;
+    const bool in = i < m.nx && j < m.ny;
+    const int k0 = blockIdx.z * kPhiRun, k1 = min(k0 + kPhiRun, m.nz);
+    const size_t n = (size_t)m.nx * m.ny * m.nz;
+    const int P = W + 1, at = (ty + 1) * P + tx + 1;
+    // the viscosities of plane k (mirrored into the domain) into a buffer; a row or column before the first is
+    // the first itself
+    auto plane = [&](int k, double *buf) {
+        if (!in) return;
+        const double mc = mom_mu(m, i, j, k);
+        buf[at] = mc;
+        if (ty == 0) buf[at - P] = j > 0 ? mom_mu(m, i, j - 1, k) : mc;
+        if (tx == 0) {
+            buf[at - 1] = i > 0 ? mom_mu(m, i - 1, j, k) : mc;
+            if (ty == 0) buf[0] = i > 0 || j > 0 ? mom_mu(m, i - 1, j - 1, k) : mc;
+        }
+    };
+    if (VISC) plane(k0 - 1, sh[(k0 + 2) % 3]);
+    for (int k = k0; k < k1; k++) {
+        double mc = 0, mx = 0, my = 0, mz = 0, mxy = 0, mxz = 0, myz = 0;
+        if (VISC) {
+            double *const b = sh[k % 3], *const bl = sh[(k + 2) % 3];
+            plane(k, b);
+            __syncthreads();
+            mc = b[at];
+            mx = b[at - 1];
+            my = b[at - P];
+            mxy = b[at - P - 1];
+            mz = bl[at];
+            mxz = bl[at - 1];
+            myz = bl[at - P];
+        }
+        const size_t c = ((size_t)k * m.ny + j) * m.nx + i;
+        if (!in || !MG_CK(c, c, (long long)n, CK_MOMENTUM)) continue;
+        mom_centre<0, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
+        mom_centre<1, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
+        mom_centre<2, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
+        // in cell-index order: the cell below along both axes, below along the higher axis, below along
+        // the lower axis, the cell itself
+        mom_edge<0, 1, CONV, VISC, POW2>(m, n, c, i, j, k, mc, mx, my, mxy);
+        mom_edge<0, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mc, mx, mz, mxz);
+        mom_edge<1, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mc, my, mz, myz);
     }
-    const size_t c = ((size_t)k * m.ny + j) * m.nx + i;
-    F = m.w[(6 + slot) * n + c];
-    S = m.w[(9 + slot) * n + c];
 }
 
-template <int A>
+// R of face A at cell (i, j, k) = c, i.e. from the values at c, at the cell before it along A and, for the
+// tangential axes, at c and the cell after it (edge values past the last cell lie on a high wall: zero flux
+// and shear, the wall's normal velocity and the mirrored tangential one)
+template <int A, bool CONV, bool VISC, bool POW2>
 __device__ __forceinline__ double mom_face(const MomArgs &m, size_t n, int i, int j, int k, size_t c, double beta)
 {
-    constexpr int ai = A == 0, aj = A == 1;
-    const size_t cm = c - (ai ? 1 : (aj ? (size_t)m.nx : (size_t)m.nx * m.ny));
-    double conv = __dmul_rn(__dsub_rn(m.w[A * n + c], m.w[A * n + cm]), m.ih);
-    double visc = __dsub_rn(m.w[(3 + A) * n + c], m.w[(3 + A) * n + cm]);
-    auto tangential = [&](auto bcon) {
-        constexpr int B = decltype(bcon)::value;
-        constexpr int bi = B == 0, bj = B == 1, bk = B == 2;
-        double F0, S0, F1, S1;
-        mom_edge_at<A, B>(m, n, i, j, k, F0, S0);
-        mom_edge_at<A, B>(m, n, i + bi, j + bj, k + bk, F1, S1);
-        conv = __dadd_rn(conv, __dmul_rn(__dsub_rn(F1, F0), m.ih));
-        visc = __dadd_rn(visc, __dsub_rn(S1, S0));
-    };
-    if (A == 0) {
-        tangential(std::integral_constant<int, 1>());
-        tangential(std::integral_constant<int, 2>());
-    } else if (A == 1) {
-        tangential(std::integral_constant<int, 0>());
-        tangential(std::integral_constant<int, 2>());
-    } else {
-        tangential(std::integral_constant<int, 0>());
-        tangential(std::integral_constant<int, 1>());
+    const size_t step[3] = {1, (size_t)m.nx, (size_t)m.nx * m.ny};
+    const bool last[3] = {i + 1 >= m.nx, j + 1 >= m.ny, k + 1 >= m.nz};
+    const size_t cm = c - step[A];
+    double conv = 0.0, visc = 0.0;
+    if (CONV) conv = mom_ih<POW2>(m, __dsub_rn(m.w[A * n + c], m.w[A * n + cm]));
+    if (VISC) visc = __dsub_rn(m.w[(3 + A) * n + c], m.w[(3 + A) * n + cm]);
+#pragma unroll
+    for (int B = 0; B < 3; B++) {
+        if (B == A) continue;
+        const int slot = A + B - 1;  // xy, xz, yz
+        if (CONV) {
+            const double *F = m.w + (6 + slot) * n;
+            const double F0 = F[c], F1 = last[B] ? 0.0 : F[c + step[B]];
+            conv = __dadd_rn(conv, mom_ih<POW2>(m, __dsub_rn(F1, F0)));
+        }
+        if (VISC) {
+            const double *S = m.w + (9 + slot) * n;
+            const double S0 = S[c], S1 = last[B] ? 0.0 : S[c + step[B]];
+            visc = __dadd_rn(visc, __dsub_rn(S1, S0));
+        }
     }
-    double r = m.convect ? -conv : 0.0;
-    r = __dadd_rn(r, __dmul_rn(__dmul_rn(m.inv_re, beta), __dmul_rn(visc, m.ih)));
+    double r = CONV ? neg_bits(conv) : 0.0;
+    // (without the viscous term the sum is with a zero: +0 for a zero of either sign, as r + 0)
+    if (VISC) r = __dadd_rn(r, __dmul_rn(__dmul_rn(m.inv_re, beta), mom_ih<POW2>(m, visc)));
+    else if (zero_bits(r)) r = 0.0;
     if (A == 2) r = __dsub_rn(r, m.g);
     return r;
 }
 
 // one thread per cell: R on its three low faces
+template <bool CONV, bool VISC, bool POW2>
 __global__ void k_mom_combine(MomArgs m)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
@@ -2289,9 +2328,9 @@ __global__ void k_mom_combine(MomArgs m)
     if (!MG_CK(c, c, (long long)n, CK_MOMENTUM)) return;
     const double bx = m.beta.bx[c], by = m.beta.by[c], bz = m.beta.bz[c];
     // an open face is interior (its low neighbour exists), so c - e_a is a cell
-    m.r.bx[c] = (i > 0 && pos_bits(bx)) ? mom_face<0>(m, n, i, j, k, c, bx) : 0.0;
-    m.r.by[c] = (j > 0 && pos_bits(by)) ? mom_face<1>(m, n, i, j, k, c, by) : 0.0;
-    m.r.bz[c] = (k > 0 && pos_bits(bz)) ? mom_face<2>(m, n, i, j, k, c, bz) : 0.0;
+    m.r.bx[c] = (i > 0 && pos_bits(bx)) ? mom_face<0, CONV, VISC, POW2>(m, n, i, j, k, c, bx) : 0.0;
+    m.r.by[c] = (j > 0 && pos_bits(by)) ? mom_face<1, CONV, VISC, POW2>(m, n, i, j, k, c, by) : 0.0;
+    m.r.bz[c] = (k > 0 && pos_bits(bz)) ? mom_face<2, CONV, VISC, POW2>(m, n, i, j, k, c, bz) : 0.0;
 }
 
 // out = 0.5 (a + b)   (b null: 0.5 a)
@@ -3624,6 +3663,15 @@ cudaError_t launch_rk_combine(size_t n, const LevelArrays<double> &a, const Leve
     return cudaGetLastError();
 }
 
+// blocks of the kernels that share face products along rows (k_phi_grad, k_divergence_mul, k_mom_parts):
+// W x R threads, a row rounded up to whole warps (at most kPhiW cells) by as many rows as fit
+inline void row_share_grid(Dims d, dim3 &grid, dim3 &block)
+{
+    const int W = std::min((d.nx + 31) / 32 * 32, kPhiW), R = std::max(1, std::min(kPhiThreads / W, d.ny));
+    grid = dim3((unsigned)((d.nx + W - 1) / W), (unsigned)((d.ny + R - 1) / R), (unsigned)((d.nz + kPhiRun - 1) / kPhiRun));
+    block = dim3((unsigned)W, (unsigned)R);
+}
+
 cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_air, double mu_water, double inv_re,
                                 double g, int convect, const LevelArrays<double> &beta, const LevelArrays<double> &u,
                                 const LevelArrays<double> &r, double *work, cudaStream_t s)
@@ -3632,8 +3680,7 @@ cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_a
     m.nx = d.nx;
     m.ny = d.ny;
     m.nz = d.nz;
-    m.convect = convect ? 1 : 0;
-    m.ih = 1.0 / h;
+    m.ih = scale2(1.0 / h);
     m.mu_air = mu_air;
     m.dmu = mu_water - mu_air;
     m.inv_re = inv_re;
@@ -3644,10 +3691,27 @@ cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_a
     m.r = r;
     m.w = work;
     const dim3 g2 = row_grid2(d.nx, d.ny, d.nz), blk = row_block2(d.nx);
-    note_launch();
-    k_mom_parts<<<g2, blk, 0, s>>>(m);
-    note_launch();
-    k_mom_combine<<<g2, blk, 0, s>>>(m);
+    dim3 pg, pb;
+    row_share_grid(d, pg, pb);
+    auto go = [&](auto conv, auto visc, auto pow2) {
+        constexpr bool C = decltype(conv)::value, V = decltype(visc)::value, P = decltype(pow2)::value;
+        if (C || V) {
+            note_launch();
+            k_mom_parts<C, V, P><<<pg, pb, 0, s>>>(m);
+        }
+        note_launch();
+        k_mom_combine<C, V, P><<<g2, blk, 0, s>>>(m);
+    };
+    auto go_p = [&](auto conv, auto visc) {
+        if (m.ih.ok) go(conv, visc, BoolTag<true>{});
+        else go(conv, visc, BoolTag<false>{});
+    };
+    const BoolTag<true> yes;
+    const BoolTag<false> no;
+    if (convect && inv_re != 0.0) go_p(yes, yes);
+    else if (convect) go_p(yes, no);
+    else if (inv_re != 0.0) go_p(no, yes);
+    else go(no, no, yes);
     return cudaGetLastError();
 }
 
@@ -3683,15 +3747,6 @@ cudaError_t launch_divergence_area(Dims d, double scale, const LevelArrays<doubl
     k_divergence_area<<<row_grid(d.nx, d.ny, d.nz), kRowThreads, 0, s>>>(d.nx, d.ny, d.nz, scale, mask, area, u, v,
                                                                          rhs);
     return cudaGetLastError();
-}
-
-// blocks of the kernels that share face products along rows (k_phi_grad, k_divergence_mul): W x R
-// threads, a row rounded up to whole warps (at most kPhiW cells) by as many rows as fit
-inline void row_share_grid(Dims d, dim3 &grid, dim3 &block)
-{
-    const int W = std::min((d.nx + 31) / 32 * 32, kPhiW), R = std::max(1, std::min(kPhiThreads / W, d.ny));
-    grid = dim3((unsigned)((d.nx + W - 1) / W), (unsigned)((d.ny + R - 1) / R), (unsigned)((d.nz + kPhiRun - 1) / kPhiRun));
-    block = dim3((unsigned)W, (unsigned)R);
 }
 
 cudaError_t launch_divergence_mul(Dims d, double scale, const LevelArrays<double> &L, const LevelArrays<double> &B,
