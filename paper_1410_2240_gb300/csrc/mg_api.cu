@@ -766,15 +766,17 @@ int final_status(mg_ctx *c, int status)
 }
 
 // p -= its mean over each fluid region (live cells), dead cells 0; with one region the mean is
-// dscal[S_SUM_P] / nlive from the last residual pass
-int remove_p_mean(mg_ctx *c, double *p)
+// dscal[S_SUM_P] / nlive, from the CG's last residual pass or (sum) summed here
+int remove_p_mean(mg_ctx *c, double *p, bool sum)
 {
     const Dims d = c->dims[0];
     if (c->ncomp > 1)
         CK(mg::launch_comp_center(d.n(), p, c->cc_label, c->ncomp, c->cc_sum, c->cc_cnt, p, c->partials, c->dscal,
                                   -1, -1, c->s, c->cc_part));
-    else
+    else {
+        if (sum) CK(mg::launch_sum_p(d, c->L64[0].dinv, p, c->partials, c->dscal, c->s));
         CK(mg::launch_sub_mean_p(d, c->L64[0].dinv, p, c->dscal, c->s));
+    }
     return MG_OK;
 }
 
@@ -846,7 +848,7 @@ int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st
     }
     // zero mean over each region's live cells (the cycle commutes with constant shifts, so once
     // suffices)
-    CKS(remove_p_mean(c, p));
+    CKS(remove_p_mean(c, p, true));
     CK(cudaEventRecord(c->ev1, s));
     CK(cudaEventSynchronize(c->ev1));
     if (st) {
@@ -1073,7 +1075,7 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
         // the loop top re-checks with the true residual (and restarts if needed)
     }
     (void)done;
-    if (!zeroed && (status == MG_OK || status == MG_ERR_NOT_CONVERGED)) CKS(remove_p_mean(c, p));
+    if (!zeroed && (status == MG_OK || status == MG_ERR_NOT_CONVERGED)) CKS(remove_p_mean(c, p, false));
     CK(cudaEventRecord(c->ev1, s));
     CK(cudaEventSynchronize(c->ev1));
     if (st) {

@@ -237,6 +237,8 @@ cudaError_t launch_rhs_prepare(Dims d, const double *rhs, const double *dinv, do
                                double *dscal, cudaStream_t s);
 cudaError_t launch_resid_norm(Dims d, double ih2, const LevelArrays<double> &L, const double *b, const double *p,
                               double *partials, double *dscal, cudaStream_t s);
+// dscal[S_SUM_P] = the sum of p over the live cells (launch_pcg_resid writes it too)
+cudaError_t launch_sum_p(Dims d, const double *dinv, const double *p, double *partials, double *dscal, cudaStream_t s);
 cudaError_t launch_sub_mean_p(Dims d, const double *dinv, double *p, const double *dscal, cudaStream_t s);
 // r32 / e32: the finest FP32 fields, in the layout sp
 cudaError_t launch_resid_cast(Dims d, double ih2, const LevelArrays<double> &L, const double *b, const double *p,
