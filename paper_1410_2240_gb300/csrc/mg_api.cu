@@ -542,9 +542,14 @@ int tail_start(const mg_ctx *c, const std::vector<LevelArrays<T>> &L, mg::TailAr
 // post-smoothing sweep, so this cycle's first red pass would compute the red values that stand there
 // from the same black ones: it is left out (the same iterate bit for bit, one of the finest level's
 // 2 (nu1 + nu2) passes less)
+// part: the cycle in two calls, the first making its first `stop` pre-smoothing passes alone, the second
+// the rest after those `done` (colour passes; a cycle of fused sweeps is not divided)
+struct CyclePart {
+    int done = 0, stop = -1;
+};
 template <typename T>
 int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T *p, bool zero = false,
-           bool again = false)
+           bool again = false, CyclePart part = {})
 {
     cudaStream_t s = c->s;
     const Dims d = c->dims[l];
@@ -576,36 +581,48 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     const bool alternate = c->o.pass_order == 1 && sp.half;
     int npass = 0;
     // the first pass reads no iterate when p starts at zero; otherwise clear p first
-    bool zpass = zero && !fused && c->o.nu1 >= 1;
+    const bool zpass = zero && !fused && c->o.nu1 >= 1;
     if (zero && !zpass) CK(cudaMemsetAsync(p, 0, d.n() * sizeof(T), s));
-    bool skip = again && !fused && c->o.nu1 >= 1 && c->o.nu2 >= 1;  // the first red pass
+    const bool skip = again && !fused && c->o.nu1 >= 1 && c->o.nu2 >= 1;  // the first red pass
+    // one colour pass; zp: p is zero
+    auto pass = [&](int colour, bool zp) -> int {
+        if (sp.half) {
+            if constexpr (std::is_same<T, float>::value)
+                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, colour, s, urow, arow, alternate ? (npass + 1) & 1 : 0, zp,
+                                           &c->sf0));
+        } else {
+            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, colour, s, zp, rec));
+        }
+        npass++;
+        return MG_OK;
+    };
     // one red-black sweep, `first` colour first
     auto sweep = [&](int first) -> int {
         ProfScope ps(c, MG_PROF_SMOOTH, fine);
-        if (fused) {
-            if (tma_level<T>(c, l))
-                CK(launch_sweep_tma(d, h2, L[l], b, cur, alt, first, c->dscal, s));
-            else
-                CK(mg::launch_rb_sweep<T>(d, h2, L[l], b, cur, alt, first, s));
-            std::swap(cur, alt);
-        } else if (sp.half) {
-            if constexpr (std::is_same<T, float>::value) {
-                const int r0 = alternate ? (npass + 1) & 1 : 0;
-                if (!skip)
-                    CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first, s, urow, arow, r0, zpass, &c->sf0));
-                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, first ^ 1, s, urow, arow,
-                                           skip ? r0 : r0 ^ (alternate ? 1 : 0), false, &c->sf0));
-                npass += skip ? 1 : 2;
-            }
-        } else {
-            if (!skip) CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first, s, zpass, rec));
-            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, first ^ 1, s, false, rec));
+        if (!fused) {
+            CKS(pass(first, false));
+            return pass(first ^ 1, false);
         }
-        zpass = false;
-        skip = false;
+        if (tma_level<T>(c, l))
+            CK(launch_sweep_tma(d, h2, L[l], b, cur, alt, first, c->dscal, s));
+        else
+            CK(mg::launch_rb_sweep<T>(d, h2, L[l], b, cur, alt, first, s));
+        std::swap(cur, alt);
         return MG_OK;
     };
-    for (int it = 0; it < c->o.nu1; it++) CKS(sweep(0));
+    for (int it = 0; it < c->o.nu1; it++) {
+        if (fused) {
+            CKS(sweep(0));
+            continue;
+        }
+        ProfScope ps(c, MG_PROF_SMOOTH, fine);
+        for (int colour = 0; colour < 2; colour++) {
+            const int m = 2 * it + colour;
+            if (m < part.done) npass++;
+            else if ((m > 0 || !skip) && (part.stop < 0 || m < part.stop)) CKS(pass(colour, m == 0 && zpass));
+        }
+    }
+    if (part.stop >= 0) return MG_OK;
     const LevelArrays<T> &C = L[l + 1];
     {
         ProfScope ps(c, MG_PROF_RESTRICT, fine);
@@ -685,6 +702,18 @@ int read_scalars(mg_ctx *c)
 {
     CK(cudaMemcpyAsync(c->hscal, c->dscal, mg::S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, c->s));
     CK(cudaStreamSynchronize(c->s));
+    return check_scalars(c);
+}
+// the same in two steps, with work queued between them that the host does not wait for
+int queue_scalars(mg_ctx *c)
+{
+    CK(cudaMemcpyAsync(c->hscal, c->dscal, mg::S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+    CK(cudaEventRecord(c->ev_h, c->s));
+    return MG_OK;
+}
+int wait_scalars(mg_ctx *c)
+{
+    CK(cudaEventSynchronize(c->ev_h));
     return check_scalars(c);
 }
 
@@ -985,16 +1014,35 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
     double rel = 0.0, nb2 = 0.0;
     bool done = false, zeroed = false;
     // precondition: z = M r (FP64) or e_cur = M (r / scale) (mixed); M = V-cycles, or the inverse
-    // diagonal of A (Jacobi: -h^2 dinv)
-    auto precondition = [&]() -> int {
+    // diagonal of A (Jacobi: -h^2 dinv); `done` passes of its first cycle are queued already
+    auto precondition = [&](int done) -> int {
         if (c->o.precond == 1) {
             CK(mg::launch_jacobi(n, -c->hs[0] * c->hs[0], c->L64[0].dinv, c->kr, z, s));
         } else if (mixed) {
-            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0, v > 0));
+            for (int v = 0; v < c->o.inner_cycles; v++)
+                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1}));
         } else {
-            for (int v = 0; v < c->o.inner_cycles; v++) CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0, v > 0));
+            for (int v = 0; v < c->o.inner_cycles; v++)
+                CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1}));
         }
         return MG_OK;
+    };
+    // The first passes of the next preconditioning, queued while the host waits for the residual of the
+    // update before them: the GPU would stand idle for the copy, the host's wait and the next launch (some
+    // 13 us an iteration, a tenth of one at 64^3).  They write e_cur or z alone, which nothing reads
+    // if the iteration was the last; as many as take some 20 us (a pass moves about three values per cell
+    // at 4 TB/s), at least one.
+    int ahead = 0;
+    if (c->o.precond == 0 && !c->o.profile && c->nlev > 1 && c->o.nu1 >= 1 &&
+        (mixed ? tail_of<float>(c).first : tail_of<double>(c).first) != 0 &&
+        !(mixed ? use_fused<float>(c, 0) : use_fused<double>(c, 0))) {
+        const double pass_us = std::max(3.0, (double)n * (mixed ? 4 : 8) * 3.0 / 4e6);
+        ahead = std::max(1, std::min(2 * c->o.nu1, (int)(20.0 / pass_us)));
+    }
+    auto begin_precondition = [&]() -> int {
+        if (ahead == 0) return MG_OK;
+        if (mixed) return vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, true, false, CyclePart{0, ahead});
+        return vcycle<double>(c, c->L64, 0, c->kr, z, true, false, CyclePart{0, ahead});
     };
     while (!done) {
         // (re)start: true residual
@@ -1031,7 +1079,7 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
                           it, tol_user, tol);
             break;
         }
-        CKS(precondition());
+        CKS(precondition(0));
         if (mixed) {
             CK(mg::launch_pcg_dots32(n, c->L32[0].b, e_cur, nullptr, c->partials, c->dscal, sc_cur, sc_cur, -1, s));
             CK(mg::launch_pcg_dir<float>(n, e_cur, c->kd, c->dscal, sc_cur, -1, 1, s, c->split0, c->partials));
@@ -1053,11 +1101,14 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
                 CK(mg::launch_pcg_update(n, c->kd, c->kq, p, c->kr, mixed ? c->L32[0].b : nullptr, c->partials, c->dscal,
                                          sc_cur, mixed ? sc_old : -1, s, c->split0));
             }
-            CKS(read_scalars(c));
+            CKS(queue_scalars(c));
+            const bool more = it < c->o.max_cycles;
+            if (more) CKS(begin_precondition());
+            CKS(wait_scalars(c));
             rel = std::sqrt(c->hscal[mg::S_RR] / nb2);
             if (st && nhist < 256) st->resid_hist[nhist++] = rel;
-            if (rel <= tol || !std::isfinite(rel) || it >= c->o.max_cycles) break;
-            CKS(precondition());
+            if (rel <= tol || !std::isfinite(rel) || !more) break;
+            CKS(precondition(ahead));
             ProfScope ps(c, MG_PROF_KRYLOV, true);
             if (mixed) {
                 CK(mg::launch_pcg_dots32(n, c->L32[0].b, e_cur, e_old, c->partials, c->dscal, sc_cur, sc_cur, sc_old,

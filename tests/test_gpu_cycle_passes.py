@@ -137,3 +137,20 @@ def test_fp64_row_records_identical_to_loaded_faces(mgp, shape, stretched):
             ctx.vcycle(rhs, p)
         out.append(p)
     assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nu,inner", [((2, 2), 1), ((1, 1), 2), ((0, 2), 1), ((5, 1), 1)])
+@pytest.mark.parametrize("shape", [(48, 16, 24), (32, 32, 32), (16, 16, 16), (20, 16, 24)])
+def test_passes_queued_ahead_change_nothing(mgp, shape, nu, inner):
+    """A profiled solve queues every cycle after the host has read the residual before it; else
+    the first passes are queued while the host waits.  The kernels and their order are the same:
+    every bit agrees, iteration counts included, also where the cycle limit ends the solve."""
+    for prec, cycles in (("fp64", 100), ("mixed", 100), ("mixed", 3)):
+        got = []
+        for profile in (0, 1):
+            _, _, b, ctx = _setup(mgp, shape, prec=prec, krylov=1, nu1=nu[0], nu2=nu[1], inner_cycles=inner,
+                                  max_cycles=cycles, profile=profile)
+            p, st = ctx.solve(dev(b), tol=1e-10, allow_not_converged=True)
+            got.append((host(p), st.cycles, st.rel_resid))
+        assert got[0][1:] == got[1][1:], prec
+        assert np.array_equal(got[0][0], got[1][0]), prec
