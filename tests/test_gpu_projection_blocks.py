@@ -75,3 +75,47 @@ def test_residual_of_the_first_iterate(mgp, shape, krylov, prec):
         assert st.rhs_norm == pytest.approx(np.linalg.norm(b), rel=n)
         assert st.rel_resid == pytest.approx(r / np.linalg.norm(b), rel=n)
         assert np.abs(host(g) - (p - p.mean())).max() <= n * max(1.0, np.abs(p).max())
+
+
+def _stretched(shape, seed, frac):
+    nx, ny, nz = shape
+    rng = np.random.default_rng(seed)
+    w = [rng.uniform(0.5, 1.5, m) / m for m in shape]
+    f = None
+    if frac:  # open, closed and partly covered faces
+        f = [np.where(rng.random((nz, ny, nx)) < 0.5, 1.0, np.maximum(rng.uniform(-0.3, 1.0, (nz, ny, nx)), 0.0))
+             for _ in range(3)]
+    return w, f
+
+
+@pytest.mark.parametrize("frac", [False, True])
+@pytest.mark.parametrize("shape", [(128, 2, 16), (129, 3, 17), (31, 5, 33), (1, 40, 15), (200, 1, 1), (2, 130, 31)])
+def test_stretched_metrics_blocks_bit_exact(mgp, shape, frac):
+    w, f = _stretched(shape, 74, frac)
+    for interface in ("random", "wave"):
+        case = synth.small_case(*shape, seed=75, solid="none", interface=interface, fields=False)
+        beta = O.face_coeffs(case.phi, None, case.lam)
+        bo, ao = mgp.stretched_metrics(*[dev(x) for x in w], faces_dev(beta), None if f is None else faces_dev(f))
+        bi, area = O.stretched_metrics(*w, beta, f)
+        for a, b in zip(faces_host(bo) + faces_host(ao), bi + area):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("body", [False, True])
+@pytest.mark.parametrize("shape", [(264, 16, 16), (36, 20, 28), (64, 48, 24), (32, 16, 72)])
+def test_divergence_with_areas_blocks_bit_exact(mgp, shape, body):
+    """Also where a closed face's velocities are not finite: such a face carries no flux."""
+    case = synth.small_case(*shape, seed=76, solid="none", interface="wave")
+    (hx, hy, hz), f = _stretched(shape, 77, True)
+    bi, area = O.stretched_metrics(hx, hy, hz, O.face_coeffs(case.phi, None, case.lam), f)
+    v = None
+    if body:
+        rng = np.random.default_rng(9)
+        v = [rng.standard_normal(case.shape) for _ in range(3)]
+    ctx = mgp.Context(faces_dev(bi), 1.0, krylov=1, coarse_max_cells=2048)
+    ctx.set_face_areas(faces_dev(area))
+    if body:
+        ctx.set_body_velocity(faces_dev(v))
+    want = O.divergence_area(area, case.u_star, 1.0, 0.3, v)
+    u = [np.where(a > 0, x, np.inf) for a, x in zip(area, case.u_star)]
+    assert np.array_equal(host(ctx.divergence(faces_dev(u), dt=0.3)), want)
