@@ -583,6 +583,9 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     // the first pass reads no iterate when p starts at zero; otherwise clear p first
     const bool zpass = zero && !fused && c->o.nu1 >= 1;
     if (zero && !zpass) CK(cudaMemsetAsync(p, 0, d.n() * sizeof(T), s));
+    // two passes as one launch where the red values between them are not needed again
+    const bool both = zpass && !fine && c->o.nu1 >= 2 && sizeof(T) == 4;
+    const bool up = sizeof(T) == 4 && !fine && !fused && c->o.nu2 >= 1 && d.n() <= mg::kUpCells;
     const bool skip = again && !fused && c->o.nu1 >= 1 && c->o.nu2 >= 1;  // the first red pass
     // one colour pass; zp: p is zero
     auto pass = [&](int colour, bool zp) -> int {
@@ -618,6 +621,11 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
         ProfScope ps(c, MG_PROF_SMOOTH, fine);
         for (int colour = 0; colour < 2; colour++) {
             const int m = 2 * it + colour;
+            if (both && m < 2) {
+                if constexpr (std::is_same<T, float>::value)
+                    if (m == 0) CK(mg::launch_smooth_first(d, h2, L[l], b, cur, s));
+                continue;
+            }
             if (m < part.done) npass++;
             else if ((m > 0 || !skip) && (part.stop < 0 || m < part.stop)) CKS(pass(colour, m == 0 && zpass));
         }
@@ -642,12 +650,18 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     }
     {
         ProfScope ps(c, MG_PROF_PROLONG, fine);
-        if (c->o.nu2 >= 1)  // a black pass follows: the red cells alone
+        if (up) {
+            if constexpr (std::is_same<T, float>::value)
+                CK(mg::launch_prolong_black(d, h2, L[l], b, C.p, cur, s));
+        } else if (c->o.nu2 >= 1)  // a black pass follows: the red cells alone
             CK(mg::launch_prolong_red<T>(d, C.p, L[l].dinv, cur, s, sp, urow, arow));
         else
             CK(mg::launch_prolong<T>(d, C.p, L[l].dinv, cur, s, sp, urow));
     }
-    for (int it = 0; it < c->o.nu2; it++) CKS(sweep(1));
+    for (int it = 0; it < c->o.nu2; it++) {
+        if (up && it == 0) CKS(pass(0, false));
+        else CKS(sweep(1));
+    }
     if (cur != p) CK(cudaMemcpyAsync(p, cur, d.n() * sizeof(T), cudaMemcpyDeviceToDevice, s));
     return MG_OK;
 }

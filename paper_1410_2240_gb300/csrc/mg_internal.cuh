@@ -156,6 +156,12 @@ cudaError_t launch_level_f32(Dims d, const LevelArrays<double> &L, LevelArrays<f
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
                           bool zero = false, const double *rec = nullptr);
+// a cycle's first red pass from zero and the black pass after it, where a red pass follows
+cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s);
+// the prolongation of ec and the black pass after it, where a red pass follows (levels of at most kUpCells cells)
+constexpr size_t kUpCells = 262144;
+cudaError_t launch_prolong_black(Dims f, float h2, const LevelArrays<float> &L, const float *b, const float *ec, float *p,
+                                 cudaStream_t s);
 // rec[8 r ..]: {vx, vy, vzl, vzh, 1 / (2 vx + 2 vy + vzl + vzh), 1 / (vx + 2 vy + vzl + vzh), 0, 0} for an interior
 // row r = k ny + j whose x-faces (walls aside), y-faces, low and high z-faces hold one positive value
 // each, zeros for any other; the inverses are the diagonal's (k_diag_inv) inside and at the x-walls

@@ -648,6 +648,41 @@ __global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L
     p[c] = gs_update(s, bc, d, gs);
 }
 
+// The first red pass of a cycle from zero and the black pass after it in one launch (FP32 levels below the
+// finest), where another red pass follows (nu1 >= 2): that pass replaces every red value without reading it, so the first ones,
+// a product of b and the inverse diagonal each, are formed by the black cells beside them and not stored.
+// Same operations in the same order as the two passes.  These levels are bound by launches and latency:
+// FP32 32^3 2.7 us (5.1 in two launches), 64^3 3.7 (6.0), 128^3 10.2 (13.6).  FP64 levels keep the two
+// passes: 13 operations per cell instead of 8 on the unit that bounds them (the coarse-grid correction of 64^3
+// was 1.9 us faster, of 160^3 6 us slower, solves 0.1 %).
+__global__ void k_smooth_first(int nx, int ny, int nz, float h2, LevelArrays<float> L, const float *__restrict__ b,
+                               float *__restrict__ p)
+{
+    const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((j + k + 1) & 1);
+    if (i >= nx || j >= ny) return;
+    const size_t sxy = (size_t)nx * ny;
+    const size_t c = (size_t)k * sxy + (size_t)j * nx + i;
+    if (!ck_cell((long long)c, i, j, k, nx, ny, nz, CK_SMOOTH)) return;
+    const bool in[6] = {i > 0, i < nx - 1, j > 0, j < ny - 1, k > 0, k < nz - 1};
+    const size_t nb[6] = {c - 1, c + 1, c - nx, c + nx, c - sxy, c + sxy};
+    float bn[6], dn[6], beta[6];
+    const float bc = b[c], d = L.dinv[c];
+#pragma unroll
+    for (int f = 0; f < 6; f++) {
+        bn[f] = in[f] ? b[nb[f]] : 0.f;
+        dn[f] = in[f] ? L.dinv[nb[f]] : 0.f;
+        const float *a = f < 2 ? L.bx : (f < 4 ? L.by : L.bz);
+        beta[f] = in[f] ? a[(f & 1) ? nb[f] : c] : 0.f;
+    }
+    const GsScale<float> gs{h2, Scale2{}};
+    float s = gs_start(bc, gs);
+#pragma unroll
+    for (int f = 0; f < 6; f++)
+        if (in[f]) s = gs_add(beta[f], gs_update(gs_start(bn[f], gs), bn[f], dn[f], gs), s);
+    p[c] = gs_update(s, bc, d, gs);
+}
+
 // the row records of an FP64 level, one warp per row (as k_uniform_rows)
 __global__ void k_row_records64(int nx, int ny, int nz, const double *__restrict__ bx, const double *__restrict__ by,
                                 const double *__restrict__ bz, double2 *__restrict__ rec)
@@ -1497,6 +1532,84 @@ __global__ void k_prolong_red4(int nx, int ny, int nz, const float *__restrict__
             if (l1) v.y += c1;
             *reinterpret_cast<float2 *>(p + m) = v;
         }
+}
+
+// The prolongation and the black pass after it in one launch (FP32 levels below the finest).  The red
+// pass that follows replaces every red value from the black ones without reading it, so the corrected red
+// values are needed by this black pass alone: each black cell corrects its six red neighbours itself and no
+// red value is written, so no thread reads what another writes.  Along an axis the neighbour within
+// the black cell's coarse cell o is the child on the far side (its other coarse cell q), the one outside the near
+// child of the coarse cell t, so 20 of the 3 x 3 x 3 coarse values serve all six.  A dead red cell is
+// corrected too: its faces are 0.  Same operations in the same order as k_prolong_red and k_smooth.
+// These levels are bound by launches and latency (four black cells per thread, a coarse cell's, was no
+// faster than the two launches: too few warps): 32^3 3.1 us (5.4 in two launches), 64^3 4.2 us (6.1).  Every red value is
+// corrected six times, so larger levels keep the two launches: 128^3 15.6 us against 12.4, and of 80^3
+// or 96 x 80 x 80 the coarse-grid correction is 1 to 2 us slower (kUpCells lies at 64^3).
+__global__ void k_prolong_black(int nx, int ny, int nz, float h2, LevelArrays<float> L, const float *__restrict__ b,
+                                const float *__restrict__ ec, float *__restrict__ p)
+{
+    const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((j + k + 1) & 1);
+    if (i >= nx || j >= ny) return;
+    const int NX = nx / 2, NY = ny / 2, NZ = nz / 2;
+    const size_t sxy = (size_t)nx * ny;
+    const size_t c = (size_t)k * sxy + (size_t)j * nx + i;
+    // coarse indices along an axis: 0 the cell's own, 1 on its near side, 2 on its far side
+    auto index = [](int v, int n, int out[3]) {
+        const int o = v >> 1, lo = max(o - 1, 0), hi = min(o + 1, n - 1);
+        out[0] = o;
+        out[1] = (v & 1) ? hi : lo;
+        out[2] = (v & 1) ? lo : hi;
+    };
+    int X[3], Y[3], Z[3];
+    index(i, NX, X);
+    index(j, NY, Y);
+    index(k, NZ, Z);
+    if (!ck_cell((long long)c, i, j, k, nx, ny, nz, CK_PROLONG) ||
+        !MG_CK(((long long)min(Z[1], Z[2]) * NY + min(Y[1], Y[2])) * NX + min(X[1], X[2]),
+               ((long long)max(Z[1], Z[2]) * NY + max(Y[1], Y[2])) * NX + max(X[1], X[2]), (long long)NX * NY * NZ,
+               CK_PROLONG))
+        return;
+    const bool xl = i > 0, xh = i < nx - 1, yl = j > 0, yh = j < ny - 1, zl = k > 0, zh = k < nz - 1;
+    const float pxl = xl ? p[c - 1] : 0.f, pxh = xh ? p[c + 1] : 0.f;
+    const float pyl = yl ? p[c - nx] : 0.f, pyh = yh ? p[c + nx] : 0.f;
+    const float pzl = zl ? p[c - sxy] : 0.f, pzh = zh ? p[c + sxy] : 0.f;
+    const float bc = b[c], d = L.dinv[c], bxl = L.bx[c], byl = L.by[c], bzl = L.bz[c];
+    const float bxh = xh ? L.bx[c + 1] : 0.f, byh = yh ? L.by[c + nx] : 0.f, bzh = zh ? L.bz[c + sxy] : 0.f;
+    float e[3][3][3];
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int bb = 0; bb < 3; bb++)
+#pragma unroll
+            for (int m = 0; m < 3; m++)
+                if ((a == 2) + (bb == 2) + (m == 2) <= 1) e[a][bb][m] = ec[((size_t)Z[a] * NY + Y[bb]) * NX + X[m]];
+    // the correction of a neighbour along `axis` (0 x, 1 y, 2 z), inside the coarse cell or not
+    auto corr = [&](int axis, bool inside) {
+        const float w[2] = {0.75f, 0.25f};
+        float s = 0.f;
+#pragma unroll
+        for (int a = 0; a < 2; a++)
+#pragma unroll
+            for (int bb = 0; bb < 2; bb++)
+#pragma unroll
+                for (int m = 0; m < 2; m++) {
+                    const int v = axis == 0 ? m : (axis == 1 ? bb : a), u = inside ? 2 * v : 1 - v;  // (o, q) or (t, o)
+                    s = fmaf(w[a] * w[bb] * w[m], e[axis == 2 ? u : a][axis == 1 ? u : bb][axis == 0 ? u : m], s);
+                }
+        return s;
+    };
+    const float xi = corr(0, true), xo = corr(0, false), yi = corr(1, true), yo = corr(1, false), zi = corr(2, true),
+                zo = corr(2, false);
+    const bool ox = i & 1, oy = j & 1, oz = k & 1;  // the inside neighbour is the lower one
+    float s = 0.f;
+    if (xl) s = fmaf(bxl, pxl + (ox ? xi : xo), s);
+    if (xh) s = fmaf(bxh, pxh + (ox ? xo : xi), s);
+    if (yl) s = fmaf(byl, pyl + (oy ? yi : yo), s);
+    if (yh) s = fmaf(byh, pyh + (oy ? yo : yi), s);
+    if (zl) s = fmaf(bzl, pzl + (oz ? zi : zo), s);
+    if (zh) s = fmaf(bzh, pzh + (oz ? zo : zi), s);
+    p[c] = d * fmaf(-h2, bc, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -3411,6 +3524,23 @@ template cudaError_t launch_smooth<double>(Dims, double, const LevelArrays<doubl
                                            cudaStream_t, bool, const double *);
 template cudaError_t launch_smooth<float>(Dims, float, const LevelArrays<float> &, const float *, float *, int,
                                           cudaStream_t, bool, const double *);
+
+cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s)
+{
+    note_launch();
+    const dim3 g = row_grid2((d.nx + 1) / 2, d.ny, d.nz), blk = row_block2((d.nx + 1) / 2);
+    k_smooth_first<<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, h2, L, b, p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prolong_black(Dims f, float h2, const LevelArrays<float> &L, const float *b, const float *ec, float *p,
+                                 cudaStream_t s)
+{
+    note_launch();
+    const dim3 g = row_grid2(f.nx / 2, f.ny, f.nz), blk = row_block2(f.nx / 2);
+    k_prolong_black<<<g, blk, 0, s>>>(f.nx, f.ny, f.nz, h2, L, b, ec, p);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_row_records64(Dims d, const LevelArrays<double> &L, double *rec, cudaStream_t s)
 {

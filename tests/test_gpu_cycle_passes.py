@@ -154,3 +154,23 @@ def test_passes_queued_ahead_change_nothing(mgp, shape, nu, inner):
             got.append((host(p), st.cycles, st.rel_resid))
         assert got[0][1:] == got[1][1:], prec
         assert np.array_equal(got[0][0], got[1][0]), prec
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (3, 1), (1, 2), (2, 0)])
+@pytest.mark.parametrize("shape", [(64, 48, 40), (36, 32, 32), (128, 16, 32), (20, 16, 24), (64, 64, 64)])
+def test_joined_coarse_passes_identical_to_fused_sweeps(mgp, shape, nu):
+    """Coarse levels whose first red and black passes, and whose prolongation and the black pass after
+    it, are one launch each: bit for bit the fused sweeps, which store every red value between."""
+    case = synth.small_case(*shape, solid="ellipsoid", seed=55)
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    rhs = dev(case.rhs)
+    for prec in ("fp64", "mixed"):
+        out = []
+        for sm in (1, 2):
+            ctx = mgp.Context(beta, case.h, prec=prec, smoother=sm, coarse_max_cells=2048, coarse_tail=0, nu1=nu[0],
+                              nu2=nu[1])
+            p = torch.zeros_like(rhs)
+            for _ in range(2):
+                ctx.vcycle(rhs, p)
+            out.append(p)
+        assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1]), prec
