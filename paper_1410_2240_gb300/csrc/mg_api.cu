@@ -98,7 +98,9 @@ struct mg_ctx {
     LevelArrays<double> rk_b1, rk_b2, rk_ut, rk_us, rk_r;
     double *rk_phis = nullptr;
     double *rk_work = nullptr;  // the momentum terms' per-cell fluxes and stresses
-    double *rec64 = nullptr;  // row records of the finest level's FP64 sweeps (MG_FP64, colour passes)
+    // row records of the levels whose colour passes take them (null elsewhere; rec_level)
+    std::vector<double *> rec64;
+    std::vector<float *> rec32;
     float *urow0 = nullptr;  // uniform-row values of the finest FP32 level (with split0)
     // banded-row records of the finest FP32 level (with split0 and nx % 8 == 0), the two row
     // counts of the last hierarchy build, and whether its sweeps use the records (more banded
@@ -454,6 +456,13 @@ const TailPlan<float> &tail_of<float>(const mg_ctx *c) { return c->tail32; }
 bool fused_level(const Dims &d) { return d.nx >= 32 && d.ny >= 8 && d.nz >= 8; }
 
 template <typename T>
+const T *rec_of(const mg_ctx *c, int l);
+template <>
+const double *rec_of<double>(const mg_ctx *c, int l) { return c->rec64.empty() ? nullptr : c->rec64[l]; }
+template <>
+const float *rec_of<float>(const mg_ctx *c, int l) { return c->rec32.empty() ? nullptr : c->rec32[l]; }
+
+template <typename T>
 bool use_fused(const mg_ctx *c, int l)
 {
     if (!fused_level(c->dims[l]) || l == c->nlev - 1) return false;
@@ -572,7 +581,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     const mg::Split sp = (sizeof(T) == 4 && l == 0) ? c->split0 : mg::Split{};
     const float *urow = (sizeof(T) == 4 && l == 0) ? c->urow0 : nullptr;
     const float4 *arow = (sizeof(T) == 4 && l == 0 && c->banded) ? c->arow0 : nullptr;
-    const double *rec = (sizeof(T) == 8 && l == 0) ? c->rec64 : nullptr;
+    const T *rec = rec_of<T>(c, l);
     T *cur = p, *alt = palt_of<T>(c, l);
     // plane order of the finest colour passes (pass_order = 1): each group of passes alternates
     // descending, ascending, ... so that every pass starts on the planes its predecessor (or the
@@ -941,12 +950,15 @@ int compute_hierarchy(mg_ctx *c, const double *const face_coeffs[3])
         CK(cudaMemcpyAsync(hcb + (size_t)a * nc, src[a], nc * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(c->hscal, c->dscal, mg::S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaEventRecord(c->ev_h, s));
-    if (c->rec64) CK(mg::launch_row_records64(c->dims[0], c->L64[0], c->rec64, s));
+    for (size_t l = 0; l < c->rec64.size(); l++)
+        if (c->rec64[l]) CK(mg::launch_row_records<double>(c->dims[l], c->L64[l], c->rec64[l], s));
     if (c->o.prec == MG_MIXED) {
         // narrowed faces and 1/sum of them (the value the FP32 smoothers form on the fly); the
         // finest level's faces also in the colour-split layout
         for (int l = 0; l < c->nlev; l++)
             CK(mg::launch_level_f32(c->dims[l], c->L64[l], c->L32[l], s, l == 0 ? &c->sf0 : nullptr, c->split0));
+        for (size_t l = 0; l < c->rec32.size(); l++)
+            if (c->rec32[l]) CK(mg::launch_row_records<float>(c->dims[l], c->L32[l], c->rec32[l], s));
         if (c->rowcnt) CK(cudaMemsetAsync(c->rowcnt, 0, 2 * sizeof(unsigned), s));
         if (c->urow0)
             CK(mg::launch_uniform_rows(c->dims[0], c->L32[0].bx, c->L32[0].by, c->L32[0].bz, c->urow0, s, c->arow0,
@@ -1282,8 +1294,14 @@ int mg_setup(mg_ctx **out, const mg_grid *g, const double *const face_coeffs[3],
         cudaGetLastError();
         return bail(fail(MG_ERR_CUDA, "mg_setup: pinned buffer / event creation failed"));
     }
-    if (c->o.prec == MG_FP64 && c->o.smoother <= 1 && c->nlev >= 2) {
-        st = c->alloc(&c->rec64, 8 * (size_t)c->dims[0].ny * c->dims[0].nz);
+    if (c->o.smoother <= 1) {
+        auto records = [&](auto &rec, int first, size_t cells) {
+            rec.resize(c->nlev, nullptr);
+            for (int l = first; l + 1 < c->nlev && st == MG_OK; l++)
+                if (l == 0 || c->dims[l].n() >= cells) st = c->alloc(&rec[l], 8 * (size_t)c->dims[l].ny * c->dims[l].nz);
+        };
+        if (c->o.prec == MG_FP64) records(c->rec64, 0, mg::kRecCells64);
+        else records(c->rec32, 1, mg::kRecCells32);
         if (st != MG_OK) return bail(st);
     }
     if (c->o.prec == MG_MIXED) {

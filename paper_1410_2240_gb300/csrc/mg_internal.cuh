@@ -155,17 +155,23 @@ cudaError_t launch_level_f32(Dims d, const LevelArrays<double> &L, LevelArrays<f
 // rec (FP64, optional): the level's row records (launch_row_records64)
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          bool zero = false, const double *rec = nullptr);
+                          bool zero = false, const T *rec = nullptr);
 // a cycle's first red pass from zero and the black pass after it, where a red pass follows
 cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s);
 // the prolongation of ec and the black pass after it, where a red pass follows (levels of at most kUpCells cells)
 constexpr size_t kUpCells = 262144;
+// Cells of a level below the finest at least, for its colour passes to take row records: where a pass that loads every
+// face (56 bytes per cell in FP64, 24 in FP32) no longer runs from L2.  Coarse-grid correction with records on the first
+// coarse level against without, us: FP32 2.1 to 3.1 M cells 105 and 104, 142 and 141, 143 and 143, 3.7 M 156 and 164,
+// 4.2 M 159 and 185, 8.4 M 294 and 361; FP64 0.5 to 1.6 M no difference, 2.1 M 244 and 252, 3.1 M 341 and 374.
+constexpr size_t kRecCells64 = 2000000, kRecCells32 = 3500000;
 cudaError_t launch_prolong_black(Dims f, float h2, const LevelArrays<float> &L, const float *b, const float *ec, float *p,
                                  cudaStream_t s);
 // rec[8 r ..]: {vx, vy, vzl, vzh, 1 / (2 vx + 2 vy + vzl + vzh), 1 / (vx + 2 vy + vzl + vzh), 0, 0} for an interior
 // row r = k ny + j whose x-faces (walls aside), y-faces, low and high z-faces hold one positive value
 // each, zeros for any other; the inverses are the diagonal's (k_diag_inv) inside and at the x-walls
-cudaError_t launch_row_records64(Dims d, const LevelArrays<double> &L, double *rec, cudaStream_t s);
+template <typename T>
+cudaError_t launch_row_records(Dims d, const LevelArrays<T> &L, T *rec, cudaStream_t s);
 // one colour of a red-black sweep on the colour-split layout (FP32, all dims even); urow (optional):
 // the level's uniform-row values, arow (optional, nx % 8 == 0, replaces urow in the sweep): its
 // banded-row records (launch_uniform_rows); rev: blocks take the planes in descending order; S

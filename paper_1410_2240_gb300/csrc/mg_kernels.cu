@@ -587,15 +587,16 @@ __device__ __forceinline__ float gs_update(float s, float b, float d, const GsSc
 
 // ZERO: the iterate is zero (the first pass of a cycle from a zero guess): the products with it are
 // zeros, so only b and the inverse diagonal are read.  Both precisions take 1/sum from dinv (in FP32 the
-// hierarchy stores exactly inv_diag's value).  ROWS (FP64 finest level): rows with a record
-// (launch_row_records64) take the faces and the inverse diagonal from it, the same values: 24 bytes per
-// cell and pass instead of 56, since a pass that loads the faces is bound by HBM (0.139 ms at 256^3) as
+// hierarchy stores exactly inv_diag's value).  ROWS (the finest FP64 level, and coarse levels from kRecCells64 and
+// kRecCells32 cells on): rows with a record (launch_row_records) take the faces and the inverse diagonal from it, the
+// same values: in FP64 24 bytes per cell and pass instead of 56, since a pass that loads the faces is bound by HBM (0.139 ms at 256^3) as
 // much as by the FP64 unit (0.132 ms at 8 operations, 0.115 at 7).  Sweep at 256^3, FP64: 0.271 ms with
 // 8 operations and every face loaded, 0.257 with 7 and the short zero pass, 0.231 with the records
 // too (the average over the passes of a cycle from zero); 128^3 40.6 -> 34.2 us.
+// FP32, a coarse level of 512 x 256 x 128: 54.6 us per pass.
 template <typename T, bool ZERO, bool ROWS>
 __global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L, const T *__restrict__ b,
-                         T *__restrict__ p, int colour, const double2 *__restrict__ rec)
+                         T *__restrict__ p, int colour, const T *__restrict__ rec)
 {
     const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
     const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((j + k + colour) & 1);
@@ -615,17 +616,18 @@ __global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L
     const T pzl = zl ? p[c - sxy] : T(0), pzh = zh ? p[c + sxy] : T(0);
     T bxl, bxh, byl, byh, bzl, bzh, d;
     bool loaded = false;
-    if constexpr (ROWS && sizeof(T) == 8) {
-        const double2 *r = rec + 4 * ((size_t)k * ny + j);
-        const double2 v0 = r[0];
+    if constexpr (ROWS) {
+        using V2 = std::conditional_t<sizeof(T) == 8, double2, float2>;
+        const T *r = rec + 8 * ((size_t)k * ny + j);
+        const V2 v0 = *reinterpret_cast<const V2 *>(r);
         if (!zero_bits(v0.x)) {
-            const double2 v1 = r[1];
+            const V2 v1 = *reinterpret_cast<const V2 *>(r + 2);
             bxl = bxh = v0.x;
             byl = byh = v0.y;
             bzl = v1.x;
             bzh = v1.y;
             // an address, not a branch: lanes apart at a wall would run the update's last product twice
-            d = reinterpret_cast<const double *>(r)[xl && xh ? 4 : 5];
+            d = r[xl && xh ? 4 : 5];
             loaded = true;
         }
     }
@@ -683,23 +685,24 @@ __global__ void k_smooth_first(int nx, int ny, int nz, float h2, LevelArrays<flo
     p[c] = gs_update(s, bc, d, gs);
 }
 
-// the row records of an FP64 level, one warp per row (as k_uniform_rows)
-__global__ void k_row_records64(int nx, int ny, int nz, const double *__restrict__ bx, const double *__restrict__ by,
-                                const double *__restrict__ bz, double2 *__restrict__ rec)
+// the row records of a level, one warp per row (as k_uniform_rows)
+template <typename T>
+__global__ void k_row_records(int nx, int ny, int nz, const T *__restrict__ bx, const T *__restrict__ by,
+                              const T *__restrict__ bz, T *__restrict__ rec)
 {
     const int lane = threadIdx.x & 31, r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (r >= ny * nz) return;
     const int j = r % ny, k = r / ny;
     const size_t sxy = (size_t)nx * ny, c0 = (size_t)r * nx;
     const bool inner = nx > 1 && j > 0 && k > 0 && j < ny - 1 && k < nz - 1;
-    double vx = 0.0, vy = 0.0, vzl = 0.0, vzh = 0.0;
+    T vx = T(0), vy = T(0), vzl = T(0), vzh = T(0);
     if (inner) {
         vx = bx[c0 + 1];
         vy = by[c0];
         vzl = bz[c0];
         vzh = bz[c0 + sxy];
     }
-    bool ok = inner && pos_bits(vx) && pos_bits(vy) && pos_bits(vzl) && pos_bits(vzh);
+    bool ok = inner && pos_bits((double)vx) && pos_bits((double)vy) && pos_bits((double)vzl) && pos_bits((double)vzh);
     if (ok)  // warp-uniform
         for (int i = lane; i < nx; i += 32) {
             const size_t c = c0 + i;
@@ -709,14 +712,18 @@ __global__ void k_row_records64(int nx, int ny, int nz, const double *__restrict
         }
     ok = __all_sync(0xffffffffu, ok);
     if (lane != 0) return;
-    double i6 = 0.0, i5 = 0.0;
+    T *r8 = rec + 8 * (size_t)r;
+    T i6 = T(0), i5 = T(0);
     if (ok) {
-        i6 = div_call(1.0, ((((vx + vx) + vy) + vy) + vzl) + vzh);
-        i5 = div_call(1.0, (((vx + vy) + vy) + vzl) + vzh);
+        i6 = div_call(T(1), ((((vx + vx) + vy) + vy) + vzl) + vzh);
+        i5 = div_call(T(1), (((vx + vy) + vy) + vzl) + vzh);
     }
-    rec[4 * (size_t)r] = ok ? make_double2(vx, vy) : make_double2(0.0, 0.0);
-    rec[4 * (size_t)r + 1] = ok ? make_double2(vzl, vzh) : make_double2(0.0, 0.0);
-    rec[4 * (size_t)r + 2] = make_double2(i6, i5);
+    r8[0] = ok ? vx : T(0);
+    r8[1] = ok ? vy : T(0);
+    r8[2] = ok ? vzl : T(0);
+    r8[3] = ok ? vzh : T(0);
+    r8[4] = i6;
+    r8[5] = i5;
 }
 
 // Colour-split layout (Split in mg_internal.cuh): slot of natural cell c in a row of parity
@@ -3509,21 +3516,20 @@ cudaError_t launch_restrict_coeffs(Dims f, const double *bx, const double *by, c
 
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          bool zero, const double *rec)
+                          bool zero, const T *rec)
 {
     note_launch();
     const dim3 g = row_grid2((d.nx + 1) / 2, d.ny, d.nz), blk = row_block2((d.nx + 1) / 2);
     const GsScale<T> gs = gs_scale<T>(h2);
-    const double2 *r2 = reinterpret_cast<const double2 *>(rec);
     if (zero) k_smooth<T, true, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
-    else if (sizeof(T) == 8 && rec) k_smooth<T, false, sizeof(T) == 8><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, r2);
+    else if (rec) k_smooth<T, false, true><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, rec);
     else k_smooth<T, false, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
     return cudaGetLastError();
 }
 template cudaError_t launch_smooth<double>(Dims, double, const LevelArrays<double> &, const double *, double *, int,
                                            cudaStream_t, bool, const double *);
 template cudaError_t launch_smooth<float>(Dims, float, const LevelArrays<float> &, const float *, float *, int,
-                                          cudaStream_t, bool, const double *);
+                                          cudaStream_t, bool, const float *);
 
 cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s)
 {
@@ -3542,14 +3548,16 @@ cudaError_t launch_prolong_black(Dims f, float h2, const LevelArrays<float> &L, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_records64(Dims d, const LevelArrays<double> &L, double *rec, cudaStream_t s)
+template <typename T>
+cudaError_t launch_row_records(Dims d, const LevelArrays<T> &L, T *rec, cudaStream_t s)
 {
     const int rows = d.ny * d.nz, warps = 8;
     note_launch();
-    k_row_records64<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(d.nx, d.ny, d.nz, L.bx, L.by, L.bz,
-                                                                       reinterpret_cast<double2 *>(rec));
+    k_row_records<T><<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(d.nx, d.ny, d.nz, L.bx, L.by, L.bz, rec);
     return cudaGetLastError();
 }
+template cudaError_t launch_row_records<double>(Dims, const LevelArrays<double> &, double *, cudaStream_t);
+template cudaError_t launch_row_records<float>(Dims, const LevelArrays<float> &, float *, cudaStream_t);
 
 cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, int colour,
                                 cudaStream_t s, const float *urow, const float4 *arow, int rev, bool zero,
