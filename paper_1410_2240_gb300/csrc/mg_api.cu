@@ -106,6 +106,7 @@ struct mg_ctx {
     // counts of the last hierarchy build, and whether its sweeps use the records (more banded
     // rows than uniform ones: a stretched grid)
     float4 *arow0 = nullptr;
+    float2 *uinv0 = nullptr;  // the inverse diagonals of the rows with a record, inside and at an x-wall
     unsigned *rowcnt = nullptr;
     // the finest FP32 face arrays in the colour-split layout (with split0 and nx % 8 == 0), read
     // by the colour passes on rows without a record
@@ -581,6 +582,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     const mg::Split sp = (sizeof(T) == 4 && l == 0) ? c->split0 : mg::Split{};
     const float *urow = (sizeof(T) == 4 && l == 0) ? c->urow0 : nullptr;
     const float4 *arow = (sizeof(T) == 4 && l == 0 && c->banded) ? c->arow0 : nullptr;
+    const float2 *uinv = (sizeof(T) == 4 && l == 0) ? c->uinv0 : nullptr;
     const T *rec = rec_of<T>(c, l);
     T *cur = p, *alt = palt_of<T>(c, l);
     // plane order of the finest colour passes (pass_order = 1): each group of passes alternates
@@ -600,7 +602,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
     auto pass = [&](int colour, bool zp) -> int {
         if (sp.half) {
             if constexpr (std::is_same<T, float>::value)
-                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, colour, s, urow, arow, alternate ? (npass + 1) & 1 : 0, zp,
+                CK(mg::launch_smooth_split(d, h2, L[l], b, cur, colour, s, urow, arow, uinv, alternate ? (npass + 1) & 1 : 0, zp,
                                            &c->sf0));
         } else {
             CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, colour, s, zp, rec));
@@ -961,7 +963,7 @@ int compute_hierarchy(mg_ctx *c, const double *const face_coeffs[3])
             if (c->rec32[l]) CK(mg::launch_row_records<float>(c->dims[l], c->L32[l], c->rec32[l], s));
         if (c->rowcnt) CK(cudaMemsetAsync(c->rowcnt, 0, 2 * sizeof(unsigned), s));
         if (c->urow0)
-            CK(mg::launch_uniform_rows(c->dims[0], c->L32[0].bx, c->L32[0].by, c->L32[0].bz, c->urow0, s, c->arow0,
+            CK(mg::launch_uniform_rows(c->dims[0], c->L32[0].bx, c->L32[0].by, c->L32[0].bz, c->urow0, s, c->arow0, c->uinv0,
                                        c->rowcnt));
         if (c->rowcnt) CK(cudaMemcpyAsync(hrow, c->rowcnt, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     }
@@ -1310,6 +1312,7 @@ int mg_setup(mg_ctx **out, const mg_grid *g, const double *const face_coeffs[3],
         if (st == MG_OK && c->split0.half) st = c->alloc(&c->urow0, (size_t)c->dims[0].ny * c->dims[0].nz);
         if (st == MG_OK && c->split0.half && c->dims[0].nx % 8 == 0) {
             st = c->alloc(&c->arow0, (size_t)c->dims[0].ny * c->dims[0].nz);
+            if (st == MG_OK) st = c->alloc(&c->uinv0, (size_t)c->dims[0].ny * c->dims[0].nz);
             if (st == MG_OK) st = c->alloc(&c->rowcnt, 2);
             if (st == MG_OK) st = c->alloc(&c->sf0.bx, c->dims[0].n());
             if (st == MG_OK) st = c->alloc(&c->sf0.by, c->dims[0].n());

@@ -178,6 +178,7 @@ cudaError_t launch_row_records(Dims d, const LevelArrays<T> &L, T *rec, cudaStre
 // (required where nx % 8 == 0): the face arrays of L in the colour-split layout
 cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, int colour,
                                 cudaStream_t s, const float *urow = nullptr, const float4 *arow = nullptr,
+                                const float2 *uinv = nullptr,
                                 int rev = 0, bool zero = false, const LevelArrays<float> *S = nullptr);
 // urow[k*ny + j] = v if row (j,k) is interior (0 < j < ny-1, 0 < k < nz-1) and every face around
 // it but its two x-walls equals v, else 0; arow
@@ -185,7 +186,7 @@ cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, c
 // each, else zeros; count (optional, two counters, incremented): uniform rows, banded rows that
 // are not uniform
 cudaError_t launch_uniform_rows(Dims d, const float *bx, const float *by, const float *bz, float *urow,
-                                cudaStream_t s, float4 *arow = nullptr, unsigned *count = nullptr);
+                                cudaStream_t s, float4 *arow = nullptr, float2 *uinv = nullptr, unsigned *count = nullptr);
 // FP32 fused sweep with TMA-staged planes (mg_sweep_tma.cu)
 bool tma_sweep_supported(Dims d);
 cudaError_t launch_rb_sweep_tma(Dims d, float h2, const LevelArrays<float> &L, const float *b, const float *p_old,

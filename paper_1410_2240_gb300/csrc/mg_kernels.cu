@@ -752,11 +752,12 @@ __device__ __forceinline__ int row_parity(unsigned c, const Split &sp)
 // On a grid stretched in z the metric factors differ per axis, and a row away from the interface
 // holds four values instead: vx on its x-faces, vy on its low and high y-faces, vzl on its low and
 // vzh on its high z-faces.  arow[r] (optional) = {vx, vy, vzl, vzh} for such a "banded" row, else
-// zeros; count[0] and count[1] (optional) receive the numbers of uniform rows and of banded rows
+// zeros.  uinv[r] (optional) = the inverse diagonals of such a row's cells {inside, at an x-wall} (left as it
+// is for other rows).  count[0] and count[1] (optional) receive the numbers of uniform rows and of banded rows
 // that are not uniform.
 __global__ void k_uniform_rows(int nx, int ny, int nz, const float *__restrict__ bx, const float *__restrict__ by,
                                const float *__restrict__ bz, float *__restrict__ urow, float4 *__restrict__ arow,
-                               unsigned *__restrict__ count)
+                               float2 *__restrict__ uinv, unsigned *__restrict__ count)
 {
     const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * warps + (threadIdx.x >> 5);
@@ -781,6 +782,8 @@ __global__ void k_uniform_rows(int nx, int ny, int nz, const float *__restrict__
         const bool uni = ok && bxv == byv && bzl == byv && bzh == byv;
         urow[r] = uni ? vy : 0.f;
         if (arow) arow[r] = ok ? make_float4(vx, vy, vzl, vzh) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (uinv && ok)
+            uinv[r] = make_float2(1.f / (((((vx + vx) + vy) + vy) + vzl) + vzh), 1.f / ((((vx + vy) + vy) + vzl) + vzh));
         if (count && ok) atomicAdd(&count[uni ? 0 : 1], 1u);
     }
 }
@@ -856,17 +859,23 @@ __global__ void k_smooth_split(int nx, int ny, int nz, float h2, LevelArrays<flo
 // face arrays: a cell's low faces are the own colour's slots, its high faces the low faces of its
 // +x, +y and +z neighbours, i.e. the other colour's slots of its x-neighbour (as for p), mb + hx
 // and mb + hxy; six float4 and one scalar, each value used.
+// A record's two inverse diagonals are read from uinv (k_uniform_rows), and only a row's first cell (OFF = 0) or its
+// last one (OFF = 1) can lie at an x-wall: without the two divisions and eight wall tests per thread a sweep
+// takes 53.5 us at 256^3 instead of 56.2, 192x160x224 26.3 (30.1), 320x192x128 33.1 (37.1), 128^3 14.4 (15.6).  The
+// pass waits for its loads (half of the issue slots are used): 72 % of the copy rate at 256^3.  More warps
+// in fewer registers (48, 40: spills) take 63.0 and 67.5 us.
 // ROWS: 1 where a warp lies in one row (OFF_ is then the row's offset), 0 where it may hold several
 // rows of both parities (off: this thread's; selected per value, so that the warp does not run the
 // two parities one after the other).
 template <int ROWS, int OFF_, bool BAND, bool ZERO>
 __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, const LevelArrays<float> &S,
                                             const float *__restrict__ b, float *__restrict__ p, int colour, float4 rv,
-                                            int g, int j, int k, int off, const float *__restrict__ dinv)
+                                            float2 iv, int g, int j, int k, int off, const float *__restrict__ dinv)
 {
     const int OFF = ROWS ? OFF_ : off;
     const float v = rv.x;
     const int G = nx / 8;
+    const bool wl = !OFF && g == 0, wh = OFF && g == G - 1;  // the first cell, the last cell at an x-wall
     const size_t sxy = (size_t)nx * ny, half = sxy * nz / 2, hx = nx / 2, hxy = sxy / 2;
     const size_t mb = ((size_t)k * sxy + (size_t)j * nx) / 2 + 4 * g;
     const float *__restrict__ o = p + (colour ? 0 : half);
@@ -917,31 +926,20 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
         for (int t = 0; t < 4; t++) out[t] = dd[t] * fmaf(-h2, bb[t], 0.f);
     } else if (v != 0.f) {
         // a row with a record: the diagonal is 6v, or 5v at an x-wall (the sums of inv_diag, in its
-        // order: 0 + v = v + 0 = v), so two divisions serve the thread's four cells; on a banded
-        // row the same with vx, vy, vzl, vzh in their places
+        // order: 0 + v = v + 0 = v), on a banded row the same with vx, vy, vzl, vzh in their places; both inverses
+        // come with the record
         const float vx = BAND ? rv.x : v, vy = BAND ? rv.y : v, vzl = BAND ? rv.z : v, vzh = BAND ? rv.w : v;
-        float inv6, inv5;
-        if (BAND) {
-            inv6 = 1.f / ((((((vx + vx) + vy) + vy) + vzl) + vzh));
-            inv5 = 1.f / ((((vx + vy) + vy) + vzl) + vzh);
-        } else {
-            const float s5 = (((v + v) + v) + v) + v;
-            inv6 = 1.f / (s5 + v);
-            inv5 = 1.f / s5;
-        }
 #pragma unroll
         for (int t = 0; t < 4; t++) {
-            const int i = 8 * g + 2 * t + OFF;
-            const float pxm = xm[t], pxp = xp[t];
             float s = 0.f;
-            if (i > 0) s = fmaf(vx, pxm, s);
-            if (i < nx - 1) s = fmaf(vx, pxp, s);
+            if (!(t == 0 && wl)) s = fmaf(vx, xm[t], s);
+            if (!(t == 3 && wh)) s = fmaf(vx, xp[t], s);
             s = fmaf(vy, oy0[t], s);
             s = fmaf(vy, oy1[t], s);
             s = fmaf(vzl, oz0[t], s);
             s = fmaf(vzh, oz1[t], s);
-            const float dinv = (i > 0 && i < nx - 1) ? inv6 : inv5;
-            out[t] = dinv * fmaf(-h2, bb[t], s);
+            const float d = ((t == 0 && wl) || (t == 3 && wh)) ? iv.y : iv.x;
+            out[t] = d * fmaf(-h2, bb[t], s);
         }
     } else {
         const float4 xl = *reinterpret_cast<const float4 *>(S.bx + so + mb);
@@ -958,13 +956,11 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
         const float fzl[4] = {zl.x, zl.y, zl.z, zl.w}, fzh[4] = {zh.x, zh.y, zh.z, zh.w};
 #pragma unroll
         for (int t = 0; t < 4; t++) {
-            const int i = 8 * g + 2 * t + OFF;
-            const float bxl = fxl[t], bxh = i < nx - 1 ? fxh[t] : 0.f;
+            const float bxl = fxl[t], bxh = fxh[t];  // (xe is 0 at the wall)
             const float byl = fyl[t], byh = fyh[t], bzl = fzl[t], bzh = fzh[t];
-            const float pxm = xm[t], pxp = xp[t];
             float s = 0.f;
-            if (i > 0) s = fmaf(bxl, pxm, s);
-            if (i < nx - 1) s = fmaf(bxh, pxp, s);
+            if (!(t == 0 && wl)) s = fmaf(bxl, xm[t], s);
+            if (!(t == 3 && wh)) s = fmaf(bxh, xp[t], s);
             if (j > 0) s = fmaf(byl, oy0[t], s);
             if (j < ny - 1) s = fmaf(byh, oy1[t], s);
             if (k > 0) s = fmaf(bzl, oz0[t], s);
@@ -977,7 +973,8 @@ __device__ __forceinline__ void split4_body(int nx, int ny, int nz, float h2, co
 template <bool BAND, bool ZERO, int ROWS>
 __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<float> S, const float *__restrict__ b,
                                 float *__restrict__ p, int colour, const float *__restrict__ urow,
-                                const float4 *__restrict__ arow, int rev, const float *__restrict__ dinv)
+                                const float4 *__restrict__ arow, const float2 *__restrict__ uinv, int rev,
+                                const float *__restrict__ dinv)
 {
     // rev: the blocks take the planes (and rows) in descending order, so that a pass that follows
     // an ascending one starts on the data that pass touched last (still in L2)
@@ -998,10 +995,11 @@ __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<fl
         const float v = urow ? urow[(size_t)k * ny + j] : 0.f;
         rv = make_float4(v, v, v, v);
     }
+    const float2 iv = uinv ? uinv[(size_t)k * ny + j] : make_float2(0.f, 0.f);
     const int off = (j + k + colour) & 1;
-    if (!ROWS) split4_body<0, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, off, dinv);
-    else if (off) split4_body<1, 1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 1, dinv);
-    else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, g, j, k, 0, dinv);
+    if (!ROWS) split4_body<0, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, iv, g, j, k, off, dinv);
+    else if (off) split4_body<1, 1, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, iv, g, j, k, 1, dinv);
+    else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, iv, g, j, k, 0, dinv);
 }
 
 // r = b - h^-2 sum_f beta_f (p_nb - p_c) at one fine cell (sum order x-,x+,y-,y+,z-,z+).
@@ -3560,16 +3558,16 @@ template cudaError_t launch_row_records<double>(Dims, const LevelArrays<double> 
 template cudaError_t launch_row_records<float>(Dims, const LevelArrays<float> &, float *, cudaStream_t);
 
 cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, int colour,
-                                cudaStream_t s, const float *urow, const float4 *arow, int rev, bool zero,
-                                const LevelArrays<float> *S)
+                                cudaStream_t s, const float *urow, const float4 *arow, const float2 *uinv, int rev,
+                                bool zero, const LevelArrays<float> *S)
 {
     note_launch();
     if (d.nx % 8 == 0) {  // four cells per thread
-        if (!S || !S->bx || !S->by || !S->bz) return cudaErrorInvalidValue;
+        if (!S || !S->bx || !S->by || !S->bz || (urow && !uinv)) return cudaErrorInvalidValue;
         const dim3 block = pair_block(d.nx / 8), grid = pair_grid(d.nx / 8, d.ny, d.nz, block);
         auto go = [&](auto band, auto zer, auto rows) {
             k_smooth_split4<decltype(band)::value, decltype(zer)::value, decltype(rows)::value ? 1 : 0>
-                <<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, rev, L.dinv);
+                <<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, h2, *S, b, p, colour, urow, arow, uinv, rev, L.dinv);
         };
         auto go_rows = [&](auto band, auto zer) {
             if (block.x == 32) go(band, zer, BoolTag<true>{});
@@ -3590,12 +3588,12 @@ cudaError_t launch_smooth_split(Dims d, float h2, const LevelArrays<float> &L, c
 }
 
 cudaError_t launch_uniform_rows(Dims d, const float *bx, const float *by, const float *bz, float *urow,
-                                cudaStream_t s, float4 *arow, unsigned *count)
+                                cudaStream_t s, float4 *arow, float2 *uinv, unsigned *count)
 {
     const int rows = d.ny * d.nz, warps = 8;
     note_launch();
     k_uniform_rows<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(d.nx, d.ny, d.nz, bx, by, bz, urow, arow,
-                                                                      count);
+                                                                      uinv, count);
     return cudaGetLastError();
 }
 
