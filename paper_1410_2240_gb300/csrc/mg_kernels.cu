@@ -188,6 +188,7 @@ struct BoolTag {
 // Kernels that share values along rows (k_face_coeffs, k_phi_grad, k_divergence_flux, k_mom_parts): blocks of at most
 // kPhiThreads threads over rows of at most kPhiW cells, kPhiRun planes per block.
 constexpr int kPhiW = 256, kPhiThreads = 512, kPhiRun = 8;
+constexpr int kMomRun = 2;  // k_mom_parts on small grids
 
 __device__ __forceinline__ bool same_bits(double a, double b)
 {
@@ -2468,17 +2469,17 @@ __device__ __forceinline__ void mom_edge(const MomArgs &m, size_t n, size_t c, i
     }
 }
 
-// blocks as k_phi_grad's (W x R threads, at most kPhiThreads, kPhiRun planes up z); the viscosities of a plane
+// blocks as k_phi_grad's (W x R threads, at most kPhiThreads, RUN planes up z); the viscosities of a plane
 // of the block, with those of the row and the column before it, in one of three buffers by plane
 // (a buffer is written again three planes later: one barrier per plane)
-template <bool CONV, bool VISC, bool POW2>
+template <bool CONV, bool VISC, bool POW2, int RUN>
 __global__ void k_mom_parts(MomArgs m)
 {
     __shared__ double sh[VISC ? 3 : 1][VISC ? kPhiThreads + kPhiW + 4 : 1];  // (R + 1) (W + 1): at most 3 x 257
     const int W = blockDim.x, R = blockDim.y, tx = threadIdx.x, ty = threadIdx.y;
     const int i = blockIdx.x * W + tx, j = blockIdx.y * R + ty;
     const bool in = i < m.nx && j < m.ny;
-    const int k0 = blockIdx.z * kPhiRun, k1 = min(k0 + kPhiRun, m.nz);
+    const int k0 = blockIdx.z * RUN, k1 = min(k0 + RUN, m.nz);
     const size_t n = (size_t)m.nx * m.ny * m.nz;
     const int P = W + 1, at = (ty + 1) * P + tx + 1;
     // the viscosities of plane k (mirrored into the domain) into a buffer; a row or column before the first is
@@ -4009,13 +4010,22 @@ cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_a
     m.r = r;
     m.w = work;
     const dim3 g2 = row_grid2(d.nx, d.ny, d.nz), blk = row_block2(d.nx);
+    // Blocks of kPhiRun planes; on a grid that makes fewer than one block per SM so, of two planes and fewer rows:
+    // both passes 32^3 29 us (72 in blocks of eight planes), 48^3 39 (92), 64^3 66 (90).  At 96^3 (240 blocks) the longer
+    // runs are the faster ones, 223 us against 238: an edge is formed again at each end of a run.
     dim3 pg, pb;
     row_share_grid(d, pg, pb);
+    const bool few = (size_t)pg.x * pg.y * pg.z < 152;
+    for (int threads = kPhiThreads; few && threads >= 128; threads /= 2) {
+        row_share_grid(d, pg, pb, kMomRun, threads);
+        if ((size_t)pg.x * pg.y * pg.z >= 2 * 152) break;
+    }
     auto go = [&](auto conv, auto visc, auto pow2) {
         constexpr bool C = decltype(conv)::value, V = decltype(visc)::value, P = decltype(pow2)::value;
         if (C || V) {
             note_launch();
-            k_mom_parts<C, V, P><<<pg, pb, 0, s>>>(m);
+            if (few) k_mom_parts<C, V, P, kMomRun><<<pg, pb, 0, s>>>(m);
+            else k_mom_parts<C, V, P, kPhiRun><<<pg, pb, 0, s>>>(m);
         }
         note_launch();
         k_mom_combine<C, V, P><<<g2, blk, 0, s>>>(m);

@@ -33,3 +33,11 @@ def test_momentum_blocks_bit_exact(mgp, shape, inv_re, convection):
     R_g = mgp.momentum_rhs(dev(case.phi), faces_dev(beta), faces_dev(case.u_star), case.h, f)
     for a, b in zip(faces_host(R_g), R_o):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(256, 40, 61), (256, 38, 64)])
+def test_momentum_long_and_short_runs_bit_exact(mgp, shape):
+    """160 blocks of eight planes (long runs) and 152 of them; one row pair less takes the short runs
+    that the smaller shapes above take."""
+    for sh in (shape, (shape[0], shape[1] - 2, shape[2])):
+        test_momentum_blocks_bit_exact(mgp, sh, 0.37, True)
