@@ -553,9 +553,11 @@ int tail_start(const mg_ctx *c, const std::vector<LevelArrays<T>> &L, mg::TailAr
 // from the same black ones: it is left out (the same iterate bit for bit, one of the finest level's
 // 2 (nu1 + nu2) passes less)
 // part: the cycle in two calls, the first making its first `stop` pre-smoothing passes alone, the second
-// the rest after those `done` (colour passes; a cycle of fused sweeps is not divided)
+// the rest after those `done` (colour passes; a cycle of fused sweeps is not divided); gate: for the first call's
+// passes from an iterate (FP64, natural layout)
 struct CyclePart {
     int done = 0, stop = -1;
+    mg::Gate gate = {};
 };
 template <typename T>
 int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T *p, bool zero = false,
@@ -605,7 +607,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
                 CK(mg::launch_smooth_split(d, h2, L[l], b, cur, colour, s, urow, arow, uinv, alternate ? (npass + 1) & 1 : 0, zp,
                                            &c->sf0));
         } else {
-            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, colour, s, zp, rec));
+            CK(mg::launch_smooth<T>(d, h2, L[l], b, cur, colour, s, zp, rec, part.gate));
         }
         npass++;
         return MG_OK;
@@ -834,6 +836,18 @@ int remove_p_mean(mg_ctx *c, double *p, bool sum)
     return MG_OK;
 }
 
+// Colour passes of the next cycle to queue before the host waits for a residual: the GPU would stand idle for the
+// copy, the host's wait and the next launch, some 13 us an iteration (a tenth of one at 64^3).  As many as take some
+// 20 us (a pass moves about three values per cell at 4 TB/s), at least one; none where the cycle is not
+// made of colour passes or is timed by parts.
+int passes_ahead(const mg_ctx *c)
+{
+    const bool mixed = c->o.prec == MG_MIXED;
+    if (c->o.profile || c->nlev < 2 || c->o.nu1 < 1 || (mixed ? use_fused<float>(c, 0) : use_fused<double>(c, 0))) return 0;
+    const double pass_us = std::max(3.0, (double)c->dims[0].n() * (mixed ? 4 : 8) * 3.0 / 4e6);
+    return std::max(1, std::min(2 * c->o.nu1, (int)(20.0 / pass_us)));
+}
+
 int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st)
 {
     cudaStream_t s = c->s;
@@ -871,6 +885,16 @@ int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st
     double rel = std::sqrt(c->hscal[mg::S_RR] / nb2);
     int cyc = 0, status = MG_OK;
     int nhist = 0;
+    // The next cycle's first passes, queued before the residual that decides on it is read (passes_ahead).  Mixed: they
+    // write the correction alone, which nothing reads if the iteration has ended.  FP64: they would change p, so each
+    // stores only where the squared residual norm is above `limit` (a little above tol^2 ||b||^2, so that the
+    // host goes on wherever a pass has stored); between the two the host queues them again.  A FP64 solve
+    // at 32^3 1.325 -> 1.227 ms, at 128^3 11.05 -> 10.93 ms.
+    const int ahead = passes_ahead(c);
+    const bool skipped = c->o.nu1 >= 1 && c->o.nu2 >= 1;  // the first red pass of a continued FP64 cycle
+    const int stop = ahead == 0 ? 0 : (mixed ? ahead : std::min(2 * c->o.nu1, ahead + (skipped ? 1 : 0)));
+    const double limit = tol * tol * nb2 * (1.0 + 1e-10);
+    int done = 0;  // of the next cycle's passes, those made
     while (!(rel <= tol)) {
         if (!std::isfinite(rel)) {
             status = fail(MG_ERR_NAN, "residual norm is not finite after %d cycles", cyc);
@@ -884,20 +908,28 @@ int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st
         cyc++;
         if (mixed) {
             for (int ic = 0; ic < c->o.inner_cycles; ic++)
-                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, c->L32[0].p, ic == 0, ic > 0));
+                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, c->L32[0].p, ic == 0, ic > 0, CyclePart{ic == 0 ? done : 0, -1, {}}));
             CK(mg::launch_accumulate(d, c->L64[0].dinv, c->L32[0].p, p, c->dscal, scale_slot, s, c->split0));
             std::swap(scale_slot, next_slot);
             ProfScope ps(c, MG_PROF_RESID64, true);
             CK(mg::launch_resid_cast(d, ih2, c->L64[0], c->b0, p, c->L32[0].b, c->partials, c->dscal, scale_slot,
                                      next_slot, s, c->split0));
         } else {
-            CKS(vcycle<double>(c, c->L64, 0, c->b0, p, false, cyc > 1));
+            CKS(vcycle<double>(c, c->L64, 0, c->b0, p, false, cyc > 1, CyclePart{done, -1, {}}));
+            done = 0;
             if (cyc % c->o.check_every != 0 && cyc < c->o.max_cycles) continue;
             ProfScope ps(c, MG_PROF_RESID64, true);
             CK(mg::launch_resid_norm(d, ih2, c->L64[0], c->b0, p, c->partials, c->dscal, s));
         }
-        CKS(read_scalars(c));
-        rel = std::sqrt(c->hscal[mg::S_RR] / nb2);
+        CKS(queue_scalars(c));
+        const bool more = stop > 0 && cyc < c->o.max_cycles;
+        if (more && mixed) CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, c->L32[0].p, true, false, CyclePart{0, stop, {}}));
+        else if (more)
+            CKS(vcycle<double>(c, c->L64, 0, c->b0, p, false, true, CyclePart{0, stop, mg::Gate{c->dscal + mg::S_RR, limit}}));
+        CKS(wait_scalars(c));
+        const double rr = c->hscal[mg::S_RR];
+        done = more && (mixed || (rr > limit && std::isfinite(rr))) ? stop : 0;
+        rel = std::sqrt(rr / nb2);
         if (st && nhist < 256) st->resid_hist[nhist++] = rel;
     }
     // zero mean over each region's live cells (the cycle commutes with constant shifts, so once
@@ -1048,29 +1080,20 @@ int pcg_impl(mg_ctx *c, const double *rhs, double *p, double tol_user, mg_stats 
             CK(mg::launch_jacobi(n, -c->hs[0] * c->hs[0], c->L64[0].dinv, c->kr, z, s));
         } else if (mixed) {
             for (int v = 0; v < c->o.inner_cycles; v++)
-                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1}));
+                CKS(vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1, {}}));
         } else {
             for (int v = 0; v < c->o.inner_cycles; v++)
-                CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1}));
+                CKS(vcycle<double>(c, c->L64, 0, c->kr, z, v == 0, v > 0, CyclePart{v == 0 ? done : 0, -1, {}}));
         }
         return MG_OK;
     };
-    // The first passes of the next preconditioning, queued while the host waits for the residual of the
-    // update before them: the GPU would stand idle for the copy, the host's wait and the next launch (some
-    // 13 us an iteration, a tenth of one at 64^3).  They write e_cur or z alone, which nothing reads
-    // if the iteration was the last; as many as take some 20 us (a pass moves about three values per cell
-    // at 4 TB/s), at least one.
-    int ahead = 0;
-    if (c->o.precond == 0 && !c->o.profile && c->nlev > 1 && c->o.nu1 >= 1 &&
-        (mixed ? tail_of<float>(c).first : tail_of<double>(c).first) != 0 &&
-        !(mixed ? use_fused<float>(c, 0) : use_fused<double>(c, 0))) {
-        const double pass_us = std::max(3.0, (double)n * (mixed ? 4 : 8) * 3.0 / 4e6);
-        ahead = std::max(1, std::min(2 * c->o.nu1, (int)(20.0 / pass_us)));
-    }
+    // the first passes of the next preconditioning, queued while the host waits for the residual of the update
+    // before them; they write e_cur or z alone, which nothing reads if the iteration was the last
+    const int ahead = c->o.precond == 0 ? passes_ahead(c) : 0;
     auto begin_precondition = [&]() -> int {
         if (ahead == 0) return MG_OK;
-        if (mixed) return vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, true, false, CyclePart{0, ahead});
-        return vcycle<double>(c, c->L64, 0, c->kr, z, true, false, CyclePart{0, ahead});
+        if (mixed) return vcycle<float>(c, c->L32, 0, c->L32[0].b, e_cur, true, false, CyclePart{0, ahead, {}});
+        return vcycle<double>(c, c->L64, 0, c->kr, z, true, false, CyclePart{0, ahead, {}});
     };
     while (!done) {
         // (re)start: true residual

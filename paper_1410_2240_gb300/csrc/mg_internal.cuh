@@ -27,6 +27,12 @@ struct LevelArrays {
     T *p = nullptr;                                  // correction (levels >= 1)
 };
 
+// a pass that stores only where *rr (a squared residual norm on the device) is finite and above limit; rr null: always
+struct Gate {
+    const double *rr = nullptr;
+    double limit = 0.0;
+};
+
 // Blocks of a grid-stride reduction at most (red_grid and vec_grid in mg_kernels.cu give the number).  A
 // reduction's partials buffer holds 2 * kRedBlocks doubles and, after them, the counter of the blocks that
 // have finished (kRedPartials doubles in all, the counter zero between reductions).
@@ -155,7 +161,7 @@ cudaError_t launch_level_f32(Dims d, const LevelArrays<double> &L, LevelArrays<f
 // rec (FP64, optional): the level's row records (launch_row_records64)
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          bool zero = false, const T *rec = nullptr);
+                          bool zero = false, const T *rec = nullptr, Gate gate = {});
 // a cycle's first red pass from zero and the black pass after it, where a red pass follows
 cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s);
 // the prolongation of ec and the black pass after it, where a red pass follows (levels of at most kUpCells cells)

@@ -595,10 +595,17 @@ __device__ __forceinline__ float gs_update(float s, float b, float d, const GsSc
 // 8 operations and every face loaded, 0.257 with 7 and the short zero pass, 0.231 with the records
 // too (the average over the passes of a cycle from zero); 128^3 40.6 -> 34.2 us.
 // FP32, a coarse level of 512 x 256 x 128: 54.6 us per pass.
-template <typename T, bool ZERO, bool ROWS>
+// GATE: a pass queued before the host knows whether the iteration has ended: it stores nothing unless the squared
+// residual norm *gate.rr is finite and above gate.limit (both compared as integers: not negative).
+template <typename T, bool ZERO, bool ROWS, bool GATE = false>
 __global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L, const T *__restrict__ b,
-                         T *__restrict__ p, int colour, const T *__restrict__ rec)
+                         T *__restrict__ p, int colour, const T *__restrict__ rec, Gate gate)
 {
+    bool go = true;
+    if constexpr (GATE) {
+        const long long rr = __double_as_longlong(*gate.rr);
+        go = rr > __double_as_longlong(gate.limit) && rr < 0x7ff0000000000000ll;
+    }
     const int j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
     const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((j + k + colour) & 1);
     if (i >= nx || j >= ny) return;
@@ -648,7 +655,8 @@ __global__ void k_smooth(int nx, int ny, int nz, GsScale<T> gs, LevelArrays<T> L
     if (yh) s = gs_add(byh, pyh, s);
     if (zl) s = gs_add(bzl, pzl, s);
     if (zh) s = gs_add(bzh, pzh, s);
-    p[c] = gs_update(s, bc, d, gs);
+    const T v = gs_update(s, bc, d, gs);
+    if (go) p[c] = v;
 }
 
 // The first red pass of a cycle from zero and the black pass after it in one launch (FP32 levels below the
@@ -3515,20 +3523,32 @@ cudaError_t launch_restrict_coeffs(Dims f, const double *bx, const double *by, c
 
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
-                          bool zero, const T *rec)
+                          bool zero, const T *rec, Gate gate)
 {
     note_launch();
     const dim3 g = row_grid2((d.nx + 1) / 2, d.ny, d.nz), blk = row_block2((d.nx + 1) / 2);
     const GsScale<T> gs = gs_scale<T>(h2);
-    if (zero) k_smooth<T, true, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
-    else if (rec) k_smooth<T, false, true><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, rec);
-    else k_smooth<T, false, false><<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, nullptr);
+    auto go = [&](auto zer, auto rows, auto gated) {
+        k_smooth<T, decltype(zer)::value, decltype(rows)::value, decltype(gated)::value>
+            <<<g, blk, 0, s>>>(d.nx, d.ny, d.nz, gs, L, b, p, colour, rec, gate);
+    };
+    const BoolTag<true> yes;
+    const BoolTag<false> no;
+    if (gate.rr) {  // (FP64, from an iterate)
+        if (sizeof(T) != 8 || zero) return cudaErrorInvalidValue;
+        if constexpr (sizeof(T) == 8) {
+            if (rec) go(no, yes, yes);
+            else go(no, no, yes);
+        }
+    } else if (zero) go(yes, no, no);
+    else if (rec) go(no, yes, no);
+    else go(no, no, no);
     return cudaGetLastError();
 }
 template cudaError_t launch_smooth<double>(Dims, double, const LevelArrays<double> &, const double *, double *, int,
-                                           cudaStream_t, bool, const double *);
+                                           cudaStream_t, bool, const double *, Gate);
 template cudaError_t launch_smooth<float>(Dims, float, const LevelArrays<float> &, const float *, float *, int,
-                                          cudaStream_t, bool, const float *);
+                                          cudaStream_t, bool, const float *, Gate);
 
 cudaError_t launch_smooth_first(Dims d, float h2, const LevelArrays<float> &L, const float *b, float *p, cudaStream_t s)
 {

@@ -198,3 +198,28 @@ def test_coarse_row_records_identical_to_loaded_faces(mgp, prec, shape):
         out.append(p)
         ctx.close()
     assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (1, 1), (3, 0), (1, 0)])
+@pytest.mark.parametrize("shape", [(48, 16, 24), (32, 32, 32), (20, 16, 24)])
+def test_stationary_passes_queued_ahead_change_nothing(mgp, shape, nu):
+    """As above for the stationary cycles, whose passes ahead work on p itself and must store nothing
+    once the iteration has ended: by its tolerance, its cycle limit or a residual that is not finite."""
+    for prec, inner, cycles, tol, every in (("fp64", 1, 100, 1e-9, 1), ("fp64", 1, 100, 1e-5, 2), ("fp64", 1, 4, 1e-12, 1),
+                                            ("mixed", 1, 100, 1e-9, 1), ("mixed", 2, 3, 1e-12, 1)):
+        got = []
+        for profile in (0, 1):
+            _, _, b, ctx = _setup(mgp, shape, prec=prec, krylov=0, nu1=nu[0], nu2=nu[1], inner_cycles=inner,
+                                  max_cycles=cycles, check_every=every, profile=profile)
+            p, st = ctx.solve(dev(b), tol=tol, allow_not_converged=True)
+            got.append((host(p), st.cycles, st.rel_resid))
+        assert got[0][1:] == got[1][1:], (prec, tol)
+        assert np.array_equal(got[0][0], got[1][0]), (prec, tol)
+    out = []
+    for profile in (0, 1):
+        _, _, b, ctx = _setup(mgp, shape, krylov=0, nu1=nu[0], nu2=nu[1], profile=profile)
+        p = dev(b * 1e200)  # a guess whose residual norm overflows
+        with pytest.raises(mgp.MGError):
+            ctx.solve(dev(b), p, tol=1e-9)
+        out.append(host(p))
+    assert np.array_equal(out[0], out[1], equal_nan=True)
