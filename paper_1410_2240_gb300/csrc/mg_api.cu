@@ -242,9 +242,9 @@ int coarse_inverse(int nx, int ny, int nz, double h, const double *bx, const dou
     const double ih2 = 1.0 / (h * h);
     const int dim[3] = {nx, ny, nz}, stride[3] = {1, nx, nx * ny};
     const double *face[3] = {bx, by, bz};
-    // conductance of the low face of cell c along an axis; 0 where closed or on the wall
+    // conductance of the low face of cell c along an axis; 0 where closed or on the wall (a NaN is neither)
     auto low = [&](int c, const int *idx, int ax) {
-        return idx[ax] > 0 && face[ax][c] > 0.0 ? face[ax][c] * ih2 : 0.0;
+        return idx[ax] > 0 && !(face[ax][c] <= 0.0) ? face[ax][c] * ih2 : 0.0;
     };
     // cells in an order with the longest axis slowest: pos[c] and its inverse
     int ax[3] = {0, 1, 2};
@@ -299,6 +299,7 @@ int coarse_inverse(int nx, int ny, int nz, double h, const double *bx, const dou
                     bw = std::max(bw, std::abs(pos[c] - pos[neighbour(c, f)]));
                     tr += g[c][f];
                 }
+        if (!std::isfinite(tr)) return fail(MG_ERR_ARG, "coarsest-grid operator is not finite");
         // banded S = L + a e e^T, row i at S[i * (bw + 1)], S[i][d] = S(i, i - bw + d); the cell e is the
         // best connected one
         const int ld = bw + 1;
