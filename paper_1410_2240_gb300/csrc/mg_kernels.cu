@@ -228,6 +228,11 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // clear sign bit; the coefficients, inverse diagonals and live masks it is applied to are never
 // NaN for finite input.  zero_bits(x) equals x == 0 for every x.
 __device__ __forceinline__ bool pos_bits(double x) { return __double_as_longlong(x) > 0; }
+// x > 0 for every x: a NaN is not (the sums of faces that may hold one)
+__device__ __forceinline__ bool pos_number(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
 // (from its two words: of the 64-bit pattern shifted left the compiler makes an FP64 comparison again)
 __device__ __forceinline__ bool zero_bits(double x)
 {
@@ -519,7 +524,7 @@ __global__ void k_diag_inv(int nx, int ny, int nz, int run, const T *__restrict_
         cur = nxt;
         bz_lo = bz_hi;
         T q = T(0);
-        if (pos_bits(s)) {
+        if (pos_number(s)) {
             if (!same_bits(s, s_last)) {
                 s_last = s;
                 q_last = div_call(T(1), s);

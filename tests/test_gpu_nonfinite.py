@@ -19,8 +19,8 @@ def mgp():
     return mgproj
 
 
-def _beta(mgp, shape=(16, 16, 16), solid="ellipsoid"):
-    case = synth.small_case(*shape, solid=solid, seed=61)
+def _beta(mgp):
+    case = synth.small_case(16, solid="ellipsoid", seed=61)
     return case, mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
 
 
@@ -47,3 +47,19 @@ def test_operator_that_is_not_finite_is_refused(mgp, prec, axis, bad):
     assert e.value.code == mgp.MG_ERR_ARG
     ctx.update(beta)
     assert np.array_equal(host(ctx.vcycle(rhs, torch.zeros_like(rhs))), want)
+
+
+@pytest.mark.parametrize("krylov", [0, 1])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_nan_between_coarse_faces_leaves_its_cells_without_a_diagonal(mgp, prec, krylov):
+    """A NaN on a face that no coarse level sees: the diagonal of its two cells is no positive number, so their
+    inverse is 0 (as for cells without an open face), every other one stands, and a solve reports NaN."""
+    case, beta = _beta(mgp)
+    want = host(mgp.Context(beta, case.h, prec=prec).level_array(0, 3))
+    beta[0][2, 3, 5] = float("nan")
+    ctx = mgp.Context(beta, case.h, prec=prec, krylov=krylov)
+    want[2, 3, 4:6] = 0.0
+    assert np.array_equal(host(ctx.level_array(0, 3)), want)
+    with pytest.raises(mgp.MGError) as e:
+        ctx.solve(dev(case.rhs))
+    assert e.value.code == mgp.MG_ERR_NAN
