@@ -239,6 +239,8 @@ __device__ __forceinline__ bool zero_bits(double x)
     return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
 }
 __device__ __forceinline__ bool zero_bits(float x) { return (__float_as_int(x) << 1) == 0; }
+// 0 + x: +0 for a zero of either sign
+__device__ __forceinline__ double zero_plus(double x) { return zero_bits(x) ? 0.0 : x; }
 
 // ---------------------------------------------------------------------------
 // Bounds-check build (-DMGP_CHECK).  Before its loads and stores a kernel checks that every index
@@ -2246,7 +2248,7 @@ __global__ void k_divergence(int nx, int ny, int nz, Scale2 scale, const double 
     const double bz0 = bz[c], bz1 = zh ? bz[c + sxy] : 0.0;
     const double ux0 = ux[c], ux1 = xh ? ux[c + 1] : 0.0, uy0 = uy[c], uy1 = yh ? uy[c + nx] : 0.0;
     const double uz0 = uz[c], uz1 = zh ? uz[c + sxy] : 0.0;
-    double d = pos_bits(bx1) ? ux1 : 0.0;  // (0 + ux1)
+    double d = pos_bits(bx1) ? zero_plus(ux1) : 0.0;
     if (pos_bits(bx0)) d -= ux0;
     if (pos_bits(by1)) d += uy1;
     if (pos_bits(by0)) d -= uy0;
@@ -2736,7 +2738,7 @@ __global__ void k_divergence_flux(int nx, int ny, int nz, Scale2 scale, LevelArr
             double tx_hi = 0.0, ty_hi = 0.0;
             if (i < nx - 1) tx_hi = threadIdx.x < W - 1 ? buf[0][t + 1] : flux.edge(0, c + 1);
             if (j < ny - 1) ty_hi = threadIdx.y < R - 1 ? buf[1][t + W] : flux.edge(1, c + nx);
-            double d = ox1 ? tx_hi : 0.0;  // (0 + tx_hi)
+            double d = ox1 ? zero_plus(tx_hi) : 0.0;
             if (ox0) d = __dsub_rn(d, tx);
             if (oy1) d = __dadd_rn(d, ty_hi);
             if (oy0) d = __dsub_rn(d, ty);
@@ -2841,7 +2843,7 @@ __global__ void k_phi_grad(int nx, int ny, int nz, double neg_half_drho, const d
             double tx_hi = 0.0, ty_hi = 0.0;
             if (i < nx - 1) tx_hi = threadIdx.x < W - 1 ? buf[0][t + 1] : sq_mul_call(bx[c + 1], gbx[c + 1]);
             if (j < ny - 1) ty_hi = threadIdx.y < R - 1 ? buf[1][t + W] : sq_mul_call(by[c + nx], gby[c + nx]);
-            double s = zero_bits(tx) ? 0.0 : tx;  // 0 + tx
+            double s = zero_plus(tx);
             if (i < nx - 1) s = __dadd_rn(s, tx_hi);
             s = __dadd_rn(s, ty);
             if (j < ny - 1) s = __dadd_rn(s, ty_hi);

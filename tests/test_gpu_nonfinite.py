@@ -63,3 +63,27 @@ def test_nan_between_coarse_faces_leaves_its_cells_without_a_diagonal(mgp, prec,
     with pytest.raises(mgp.MGError) as e:
         ctx.solve(dev(case.rhs))
     assert e.value.code == mgp.MG_ERR_NAN
+
+
+@pytest.mark.parametrize("areas,body", [(False, False), (True, False), (False, True), (True, True)])
+def test_divergence_of_zeros_of_either_sign(mgp, areas, body):
+    """The sum over a cell's faces starts from +0, so velocities that are zeros of either sign give the
+    zeros that the six additions and subtractions give, sign for sign."""
+    case, beta = _beta(mgp)
+    rng = np.random.default_rng(62)
+    zeros = lambda: np.where(rng.random(case.phi.shape) < 0.5, 0.0, -0.0)
+    u, v = [zeros() for _ in range(3)], [zeros() for _ in range(3)]
+    ctx = mgp.Context(beta, case.h)
+    if areas:
+        ctx.set_face_areas(tuple(dev(np.full(case.phi.shape, 0.5)) for _ in range(3)))
+    if body:
+        ctx.set_body_velocity(tuple(dev(x) for x in v))
+    got = host(ctx.divergence(tuple(dev(x) for x in u)))
+    d = np.zeros(case.phi.shape)
+    for axis, b, x, y in zip((2, 1, 0), beta, u, v):
+        flux = x - y if body else x
+        at = lambda a, lo, hi: a[tuple(slice(lo, hi) if i == axis else slice(None) for i in range(3))]
+        is_open, f = host(b) > 0, flux
+        at(d, 0, -1)[...] = np.where(at(is_open, 1, None), at(d, 0, -1) + at(f, 1, None), at(d, 0, -1))
+        d = np.where(is_open, d - f, d)
+    assert np.array_equal(got, d) and np.array_equal(np.signbit(got), np.signbit(d))
