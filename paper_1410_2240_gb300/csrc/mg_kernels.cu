@@ -2337,7 +2337,9 @@ __global__ void k_stretched_metrics(int nx, int ny, int nz, const double *__rest
     const double dx = i ? __dmul_rn(0.5, __dadd_rn(hx[i - 1], wx)) : 1.0;
     const double dy = j ? __dmul_rn(0.5, __dadd_rn(hy[j - 1], wy)) : 1.0;
     const double r0 = zref[0], r1 = zref[1];
-    double bx_last = 0.0, qx = 0.0, by_last = 0.0, qy = 0.0;  // 0 / d = 0
+    // (a NaN is its own quotient; 0 is not, where widths are not positive)
+    const double none = __longlong_as_double(0x7ff8000000000000ll);
+    double bx_last = none, qx = none, by_last = none, qy = none;
     auto area = [&](double w, double f) { return same_bits(f, 1.0) ? w : dmul_call(w, f); };
     size_t c = (size_t)k0 * sxy + (size_t)j * nx + i;
     for (int k = k0; k < k1; k++, c += sxy) {

@@ -87,3 +87,24 @@ def test_divergence_of_zeros_of_either_sign(mgp, areas, body):
         at(d, 0, -1)[...] = np.where(at(is_open, 1, None), at(d, 0, -1) + at(f, 1, None), at(d, 0, -1))
         d = np.where(is_open, d - f, d)
     assert np.array_equal(got, d) and np.array_equal(np.signbit(got), np.signbit(d))
+
+
+@pytest.mark.parametrize("shape", [(16, 12, 20), (104, 100, 100)])
+def test_stretched_metrics_divide_closed_faces_too(mgp, shape):
+    """Widths are not checked: 0 / d on a closed face is the quotient, NaN or a zero of either sign, whatever d is."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(63)
+    widths = [rng.choice([0.5, 1.0, 0.0, -1.0, float("nan")], n) for n in shape]
+    beta = [np.where(rng.random((nz, ny, nx)) < 0.5, 0.0, 2.0) for _ in range(3)]
+    got, area = mgp.stretched_metrics(*(dev(w) for w in widths), tuple(dev(b) for b in beta))
+    for a, (b, g) in enumerate(zip(beta, got)):
+        d = 0.5 * (widths[a][:-1] + widths[a][1:])
+        want = np.zeros_like(b)
+        inner = [slice(None)] * 3
+        inner[2 - a] = slice(1, None)
+        with np.errstate(all="ignore"):
+            want[tuple(inner)] = b[tuple(inner)] / d.reshape([-1 if i == 2 - a else 1 for i in range(3)])
+        g = host(g)
+        assert np.array_equal(g, want, equal_nan=True), a
+        number = ~np.isnan(want)
+        assert np.array_equal(np.signbit(g[number]), np.signbit(want[number])), a
