@@ -3747,13 +3747,9 @@ cudaError_t launch_coarse_solve(int n, const double *M, const T *b, T *e, cudaSt
                                                                                                                 e);
     return cudaGetLastError();
 }
-// a launch of k_tail on a cluster (of more than 8 CTAs by opt-in)
-template <typename T>
-cudaError_t tail_config(int ctas, size_t smem, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at)
+// a launch of k_tail on a cluster
+inline void tail_config(int ctas, size_t smem, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && ctas > 8)
-        e = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cfg = cudaLaunchConfig_t{};
     at = cudaLaunchAttribute{};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -3764,11 +3760,13 @@ cudaError_t tail_config(int ctas, size_t smem, cudaLaunchConfig_t &cfg, cudaLaun
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return e;
 }
 
 // CTAs of the largest cluster (16, else 8) that the current device holds with kTailSmem bytes each, 0 if
-// neither: a property of the device, asked once for each (the query takes some 80 us)
+// neither: a property of the device, asked once for each (the query takes some 80 us).
+// The kernel's shared-memory limit and its cluster opt-in belong to the function, so every context and thread of a
+// device shares them: they are set here, by each mg_setup before the context's first launch, always to the same values, and
+// never by a launch.  (A limit set to a context's own need fails another thread's larger launch between the two.)
 template <typename T>
 int tail_ctas()
 {
@@ -3776,19 +3774,26 @@ int tail_ctas()
     static std::atomic<int> known[kDevices];  // 1 + the answer
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    cudaError_t e = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    const bool wide = cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     if (dev < kDevices && known[dev].load() > 0) return known[dev].load() - 1;
     int n = 0;
     for (int ctas : {16, 8}) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at;
         int clusters = 0;
-        if (tail_config<T>(ctas, kTailSmem, cfg, at) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&clusters, k_tail<T>, &cfg) == cudaSuccess && clusters >= 1) {
+        tail_config(ctas, kTailSmem, cfg, at);
+        if ((wide || ctas <= 8) && cudaOccupancyMaxActiveClusters(&clusters, k_tail<T>, &cfg) == cudaSuccess &&
+            clusters >= 1) {
             n = ctas;
             break;
         }
-        cudaGetLastError();
     }
+    cudaGetLastError();
     if (dev < kDevices) known[dev].store(n + 1);
     return n;
 }
@@ -3805,8 +3810,7 @@ cudaError_t launch_tail(const TailArgs<T> &a, cudaStream_t s)
     if (a.nlev < 2 || a.nlev > kTailMaxLevels || a.ctas < 1 || a.smem > kTailSmem) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
-    const cudaError_t e = tail_config<T>(a.ctas, a.smem, cfg, at);
-    if (e != cudaSuccess) return e;
+    tail_config(a.ctas, a.smem, cfg, at);
     cfg.stream = s;
     note_launch();
     return cudaLaunchKernelEx(&cfg, k_tail<T>, a);
