@@ -2308,28 +2308,64 @@ __global__ void k_face_areas(int nx, int ny, int nz, const double *__restrict__ 
 // index grid (unit spacing): beta_idx = beta / d with d the distance between the two cell centres,
 // area = the face's two widths times the open fraction (frac, or 1); walls 0.  Each operation
 // rounded separately.
-//
-// Bound by the FP64 unit if every face divides (some 42 operations per cell).  Threads walk up z in runs of kRun
+// On small grids one thread per cell, every face divided where it stands: the launch is a round trip to memory and a
+// division long (launch_stretched_metrics has the line).
+__global__ void k_stretched_metrics_cells(int nx, int ny, int nz, const double *__restrict__ hx,
+                                          const double *__restrict__ hy, const double *__restrict__ hz,
+                                          LevelArrays<double> beta, LevelArrays<double> frac, LevelArrays<double> bout,
+                                          LevelArrays<double> aout)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    if (i >= nx || j >= ny) return;
+    const size_t c = ((size_t)k * ny + j) * nx + i;
+    if (i == 0) {
+        bout.bx[c] = 0.0;
+        aout.bx[c] = 0.0;
+    } else {
+        const double d = __dmul_rn(0.5, __dadd_rn(hx[i - 1], hx[i]));
+        bout.bx[c] = div_call(beta.bx[c], d);
+        aout.bx[c] = __dmul_rn(__dmul_rn(hy[j], hz[k]), frac.bx ? frac.bx[c] : 1.0);
+    }
+    if (j == 0) {
+        bout.by[c] = 0.0;
+        aout.by[c] = 0.0;
+    } else {
+        const double d = __dmul_rn(0.5, __dadd_rn(hy[j - 1], hy[j]));
+        bout.by[c] = div_call(beta.by[c], d);
+        aout.by[c] = __dmul_rn(__dmul_rn(hx[i], hz[k]), frac.by ? frac.by[c] : 1.0);
+    }
+    if (k == 0) {
+        bout.bz[c] = 0.0;
+        aout.bz[c] = 0.0;
+    } else {
+        const double d = __dmul_rn(0.5, __dadd_rn(hz[k - 1], hz[k]));
+        bout.bz[c] = div_call(beta.bz[c], d);
+        aout.bz[c] = __dmul_rn(__dmul_rn(hx[i], hy[j]), frac.bz ? frac.bz[c] : 1.0);
+    }
+}
+
+// On larger grids: bound by the FP64 unit if every face divides (some 42 operations per cell).  Threads walk up z in runs of RUN
 // planes: x and y distances are fixed, so a quotient is kept until beta changes; the z distance
 // changes with every plane, so the block tabulates the quotients of two values of beta_z for
 // its planes (one division of one warp), the ones found at its first cell's bottom and top, and only cells with
 // another value divide.  Areas fully open are not multiplied by 1.  192x160x224: 0.461 -> 0.178 ms.
+template <int RUN>
 __global__ void k_stretched_metrics(int nx, int ny, int nz, const double *__restrict__ hx,
                                     const double *__restrict__ hy, const double *__restrict__ hz,
                                     LevelArrays<double> beta, LevelArrays<double> frac, LevelArrays<double> bout,
                                     LevelArrays<double> aout)
 {
-    __shared__ double zq[2][kRun], zref[2];
+    __shared__ double zq[2][RUN], zref[2];
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     const int t = threadIdx.y * blockDim.x + threadIdx.x;
-    const int k0 = blockIdx.z * kRun, k1 = min(k0 + kRun, nz);
+    const int k0 = blockIdx.z * RUN, k1 = min(k0 + RUN, nz);
     const size_t sxy = (size_t)nx * ny;
-    if (t < 2 * kRun) {
+    if (t < 2 * RUN) {
         const size_t c0 = (size_t)(blockIdx.y * blockDim.y) * nx + (size_t)blockIdx.x * blockDim.x;  // the block's first cell
-        const int m = t / kRun, k = k0 + t % kRun;
+        const int m = t / RUN, k = k0 + t % RUN;
         const double r = beta.bz[c0 + (size_t)(m ? k1 - 1 : k0) * sxy];
-        if (k > 0 && k < nz) zq[m][t % kRun] = div_call(r, __dmul_rn(0.5, __dadd_rn(hz[k - 1], hz[k])));
-        if (t % kRun == 0) zref[m] = r;
+        if (k > 0 && k < nz) zq[m][t % RUN] = div_call(r, __dmul_rn(0.5, __dadd_rn(hz[k - 1], hz[k])));
+        if (t % RUN == 0) zref[m] = r;
     }
     __syncthreads();
     if (i >= nx || j >= ny) return;
@@ -2337,9 +2373,9 @@ __global__ void k_stretched_metrics(int nx, int ny, int nz, const double *__rest
     const double dx = i ? __dmul_rn(0.5, __dadd_rn(hx[i - 1], wx)) : 1.0;
     const double dy = j ? __dmul_rn(0.5, __dadd_rn(hy[j - 1], wy)) : 1.0;
     const double r0 = zref[0], r1 = zref[1];
-    // (a NaN is its own quotient; 0 is not, where widths are not positive)
-    const double none = __longlong_as_double(0x7ff8000000000000ll);
-    double bx_last = none, qx = none, by_last = none, qy = none;
+    // (0 / d is 0 where the widths are positive; they are not checked)
+    double bx_last = 0.0, qx = pos_number(dx) ? 0.0 : div_call(0.0, dx);
+    double by_last = 0.0, qy = pos_number(dy) ? 0.0 : div_call(0.0, dy);
     auto area = [&](double w, double f) { return same_bits(f, 1.0) ? w : dmul_call(w, f); };
     size_t c = (size_t)k0 * sxy + (size_t)j * nx + i;
     for (int k = k0; k < k1; k++, c += sxy) {
@@ -4010,9 +4046,23 @@ cudaError_t launch_stretched_metrics(Dims d, const double *hx, const double *hy,
                                     const LevelArrays<double> &bout, const LevelArrays<double> &aout, cudaStream_t s)
 {
     note_launch();
+    // Per cell below 600,000 cells, in runs of 4 planes below 1.2 M and of kRun above: a block walks its run one plane after the
+    // other, 30 us for 16 planes however few blocks there are.  Per cell, 4 and 16 planes (z stretched, waves; us): 16^3 4.9, 13, 32;
+    // 32^3 6, 16, 36; 64^3 23, 28, 45; 224x56x40 38, 40, 56; 80^3 45, 42, 54; 88^3 55, 48, 57; 96^3 65, 52, 61; 500x500x4 68, 65, 65;
+    // 112^3 114, 80, 92; 128^3 148, 100, 114; 192x160x224 473, 254, 211; 256^3 1143, 553, 451.
     const dim3 blk = row_block2(d.nx);
-    const dim3 grid((d.nx + blk.x - 1) / blk.x, (d.ny + blk.y - 1) / blk.y, (d.nz + kRun - 1) / kRun);
-    k_stretched_metrics<<<grid, blk, 0, s>>>(d.nx, d.ny, d.nz, hx, hy, hz, beta, frac, bout, aout);
+    auto grid = [&](int run) {
+        return dim3((d.nx + blk.x - 1) / blk.x, (d.ny + blk.y - 1) / blk.y, (d.nz + run - 1) / run);
+    };
+    auto go = [&](auto tag) {
+        constexpr int R = decltype(tag)::value;
+        k_stretched_metrics<R><<<grid(R), blk, 0, s>>>(d.nx, d.ny, d.nz, hx, hy, hz, beta, frac, bout, aout);
+    };
+    const dim3 g1 = grid(1), g4 = grid(4);  // (a grid's z extent is at most 65535)
+    if (d.n() < 600000 && g1.z <= 65535)
+        k_stretched_metrics_cells<<<g1, blk, 0, s>>>(d.nx, d.ny, d.nz, hx, hy, hz, beta, frac, bout, aout);
+    else if (d.n() < 1200000 && g4.z <= 65535) go(std::integral_constant<int, 4>{});
+    else go(std::integral_constant<int, kRun>{});
     return cudaGetLastError();
 }
 

@@ -1,0 +1,46 @@
+"""Kernels that a small grid takes cell by cell and a large one in blocks that walk up z: each side of every line,
+with rows and runs that do not fill the blocks.  Bit for bit the oracle's (the same separately rounded operations in
+the same order)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1410_2240_gb300 import synth
+
+from _gpu_util import dev, faces_dev, faces_host, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mgp():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1410_2240_gb300 import mgproj
+    return mgproj
+
+
+def _areas(shape, seed):
+    """Open, closed and partly covered faces."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(seed)
+    return [np.where(rng.random((nz, ny, nx)) < 0.5, 1.0, np.maximum(rng.uniform(-0.3, 1.0, (nz, ny, nx)), 0.0))
+            for _ in range(3)]
+
+
+@pytest.mark.parametrize("frac", [False, True])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (84, 84, 85), (85, 84, 84), (85, 85, 85), (300, 48, 49), (129, 171, 32),
+                                   (31, 685, 33), (2, 700, 501), (700, 1001, 1), (1, 3, 70001), (1, 2, 350001),
+                                   (107, 107, 105), (129, 283, 33), (1, 700, 1716)])
+def test_stretched_metrics_bit_exact_on_both_routes(mgp, shape, frac):
+    rng = np.random.default_rng(81)
+    w = [rng.uniform(0.5, 1.5, m) / m for m in shape]
+    f = _areas(shape, 82) if frac else None
+    for interface in ("random", "wave"):
+        case = synth.small_case(*shape, seed=83, solid="none", interface=interface, fields=False)
+        beta = O.face_coeffs(case.phi, None, case.lam)
+        bo, ao = mgp.stretched_metrics(*[dev(x) for x in w], faces_dev(beta), None if f is None else faces_dev(f))
+        bi, area = O.stretched_metrics(*w, beta, f)
+        for a, b in zip(faces_host(bo) + faces_host(ao), bi + area):
+            assert np.array_equal(a, b)
