@@ -2732,12 +2732,37 @@ struct FluxArea {
     }
 };
 
+// With areas or a body velocity on small grids: a thread per cell, each of its faces' fluxes formed where it stands
+// (launch_divergence_area has the lines).
+__global__ void k_divergence_area(int nx, int ny, int nz, Scale2 scale, LevelArrays<double> mask,
+                                  LevelArrays<double> area, LevelArrays<double> u, LevelArrays<double> v,
+                                  double *__restrict__ rhs)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    if (i >= nx || j >= ny) return;
+    const size_t sxy = (size_t)nx * ny;
+    const size_t c = (size_t)k * sxy + (size_t)j * nx + i;
+    if (!ck_cell((long long)c, i, j, k, nx, ny, nz, CK_DIVERGENCE)) return;
+    auto flux = [&](const double *a, const double *uu, const double *vv, size_t f) {
+        const double du = vv ? __dsub_rn(uu[f], vv[f]) : uu[f];
+        return a ? __dmul_rn(a[f], du) : du;
+    };
+    double d = 0.0;
+    if (i < nx - 1 && pos_bits(mask.bx[c + 1])) d = __dadd_rn(d, flux(area.bx, u.bx, v.bx, c + 1));
+    if (pos_bits(mask.bx[c])) d = __dsub_rn(d, flux(area.bx, u.bx, v.bx, c));
+    if (j < ny - 1 && pos_bits(mask.by[c + nx])) d = __dadd_rn(d, flux(area.by, u.by, v.by, c + nx));
+    if (pos_bits(mask.by[c])) d = __dsub_rn(d, flux(area.by, u.by, v.by, c));
+    if (k < nz - 1 && pos_bits(mask.bz[c + sxy])) d = __dadd_rn(d, flux(area.bz, u.bz, v.bz, c + sxy));
+    if (pos_bits(mask.bz[c])) d = __dsub_rn(d, flux(area.bz, u.bz, v.bz, c));
+    rhs[c] = mul_s2(d, scale);
+}
+
 // rhs_c = scale * the sum over the open faces of c (L's coefficient > 0) of +- the flux, x+ added
 // and x- subtracted, then y, then z (as k_divergence).  Blocks as k_phi_grad: each face's
 // flux formed once, the x+ and y+ ones taken from the neighbours through shared memory (formed
 // again only at the block's right edge and top row), the z+ one carried up the column.  With areas and
-// no body velocity 10 FP64 operations per cell instead of 13 (192x160x224: 0.247 -> 0.170 ms).
-template <typename F>
+// no body velocity 10 FP64 operations per cell instead of 13 (192x160x224: 0.247 -> 0.170 ms).  RUN planes per block.
+template <int RUN, typename F>
 __global__ void k_divergence_flux(int nx, int ny, int nz, Scale2 scale, LevelArrays<double> L, F flux,
                                   double *__restrict__ rhs)
 {
@@ -2746,7 +2771,7 @@ __global__ void k_divergence_flux(int nx, int ny, int nz, Scale2 scale, LevelArr
     const int i = blockIdx.x * W + threadIdx.x, j = blockIdx.y * R + threadIdx.y;
     const int t = threadIdx.y * W + threadIdx.x;
     const bool in = i < nx && j < ny;
-    const int k0 = blockIdx.z * kPhiRun, k1 = min(k0 + kPhiRun, nz);
+    const int k0 = blockIdx.z * RUN, k1 = min(k0 + RUN, nz);
     const size_t sxy = (size_t)nx * ny;
     size_t c = in ? (size_t)k0 * sxy + (size_t)j * nx + i : 0;
     const bool ok0 = in && ck_cell((long long)c, i, j, k0, nx, ny, nz, CK_DIVERGENCE);
@@ -4155,9 +4180,25 @@ cudaError_t launch_divergence_area(Dims d, double scale, const LevelArrays<doubl
                                    const LevelArrays<double> &v, double *rhs, cudaStream_t s)
 {
     note_launch();
+    const Scale2 sc = scale2(scale);
+    // Per cell below 150,000 cells, runs of two planes below 5 M and of kPhiRun above: a block walks its run one plane after the
+    // other behind a barrier each.  Per cell, 2 and 8 planes (areas, dt = 1; us): 16^3 3.5, 5.9, 18; 32^3 3.8, 5.9, 18; 512x16x16 6.5,
+    // 6.5, 20; 16x512x16 6.6, 9.1, 18; 48^3 7.7, 6.1, 18; 64^3 11, 9.1, 18; 80^3 23, 19, 28; 96^3 32, 27, 28; 128^3 73, 58, 73; 160^3
+    // 140, 112, 123; 192x160x224 230, 173, 169; 256^3 550, 422, 400.
+    if (d.n() < 150000) {
+        k_divergence_area<<<row_grid2(d.nx, d.ny, d.nz), row_block2(d.nx), 0, s>>>(d.nx, d.ny, d.nz, sc, mask, area, u, v,
+                                                                                    rhs);
+        return cudaGetLastError();
+    }
     dim3 grid, block;
-    row_share_grid(d, grid, block);
-    k_divergence_flux<<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, scale2(scale), mask, FluxArea{area, u, v}, rhs);
+    const FluxArea flux{area, u, v};
+    if (d.n() < 5000000) {
+        row_share_grid(d, grid, block, 2);
+        k_divergence_flux<2><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, sc, mask, flux, rhs);
+    } else {
+        row_share_grid(d, grid, block);
+        k_divergence_flux<kPhiRun><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, sc, mask, flux, rhs);
+    }
     return cudaGetLastError();
 }
 
@@ -4171,7 +4212,7 @@ cudaError_t launch_divergence_mul(Dims d, double scale, const LevelArrays<double
     w.bx = const_cast<double *>(wx);
     w.by = const_cast<double *>(wy);
     w.bz = const_cast<double *>(wz);
-    k_divergence_flux<<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, scale2(scale), L, FluxMul{B, w}, rhs);
+    k_divergence_flux<kPhiRun><<<grid, block, 0, s>>>(d.nx, d.ny, d.nz, scale2(scale), L, FluxMul{B, w}, rhs);
     return cudaGetLastError();
 }
 

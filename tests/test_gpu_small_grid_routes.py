@@ -44,3 +44,22 @@ def test_stretched_metrics_bit_exact_on_both_routes(mgp, shape, frac):
         bi, area = O.stretched_metrics(*w, beta, f)
         for a, b in zip(faces_host(bo) + faces_host(ao), bi + area):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("areas,body", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (16, 128, 64), (32, 64, 72), (56, 56, 48), (144, 48, 40), (264, 32, 32),
+                                   (160, 160, 192), (192, 160, 192)])
+def test_divergence_bit_exact_on_every_route(mgp, shape, areas, body):
+    case = synth.small_case(*shape, seed=84, solid="none", interface="wave", fields=False)
+    rng = np.random.default_rng(85)
+    field = lambda: [rng.standard_normal(case.shape) for _ in range(3)]
+    f = _areas(shape, 86) if areas else [np.ones(case.shape)] * 3
+    _, area = O.stretched_metrics(*[np.ones(n) for n in shape], O.face_coeffs(case.phi, None, case.lam), f)
+    u, v = field(), (field() if body else None)
+    ctx = mgp.Context(faces_dev(O.face_coeffs(case.phi, None, case.lam)), 1.0, coarse_max_cells=2048)
+    if areas:
+        ctx.set_face_areas(faces_dev(area))
+    if body:
+        ctx.set_body_velocity(faces_dev(v))
+    for dt in (1.0, 0.3):
+        assert np.array_equal(host(ctx.divergence(faces_dev(u), dt=dt)), O.divergence_area(area, u, 1.0, dt, v))
