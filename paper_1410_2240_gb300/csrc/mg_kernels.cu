@@ -188,7 +188,7 @@ struct BoolTag {
 // Kernels that share values along rows (k_face_coeffs, k_phi_grad, k_divergence_flux, k_mom_parts): blocks of at most
 // kPhiThreads threads over rows of at most kPhiW cells, kPhiRun planes per block.
 constexpr int kPhiW = 256, kPhiThreads = 512, kPhiRun = 8;
-constexpr int kMomRun = 2;  // k_mom_parts on small grids
+constexpr int kMomRun = 2;  // k_mom_parts on grids of medium size
 
 __device__ __forceinline__ bool same_bits(double a, double b)
 {
@@ -2522,13 +2522,48 @@ __device__ __forceinline__ void mom_edge(const MomArgs &m, size_t n, size_t c, i
     }
 }
 
+// the viscosities a cell's terms use: its own and those of the cells below it along x, y, z, xy, xz and yz
+struct MomMu {
+    double c, x, y, z, xy, xz, yz;
+};
+
+// the fluxes and stresses of a cell
+template <bool CONV, bool VISC, bool POW2>
+__device__ __forceinline__ void mom_cell(const MomArgs &m, size_t n, size_t c, int i, int j, int k, const MomMu &mu)
+{
+    mom_centre<0, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c);
+    mom_centre<1, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c);
+    mom_centre<2, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c);
+    // in cell-index order: the cell below along both axes, below along the higher axis, below along
+    // the lower axis, the cell itself
+    mom_edge<0, 1, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c, mu.x, mu.y, mu.xy);
+    mom_edge<0, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c, mu.x, mu.z, mu.xz);
+    mom_edge<1, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mu.c, mu.y, mu.z, mu.yz);
+}
+
+// one thread per cell, which forms the viscosities it uses itself: where there are none to share (no viscous
+// term), on small grids and on those whose rows leave the sharing blocks' lanes idle
+template <bool CONV, bool VISC, bool POW2>
+__global__ void k_mom_parts_cells(MomArgs m)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    if (i >= m.nx || j >= m.ny) return;
+    const size_t n = (size_t)m.nx * m.ny * m.nz, c = ((size_t)k * m.ny + j) * m.nx + i;
+    if (!MG_CK(c, c, (long long)n, CK_MOMENTUM)) return;
+    MomMu mu{};
+    if (VISC)
+        mu = MomMu{mom_mu(m, i, j, k),         mom_mu(m, i - 1, j, k),     mom_mu(m, i, j - 1, k),    mom_mu(m, i, j, k - 1),
+                   mom_mu(m, i - 1, j - 1, k), mom_mu(m, i - 1, j, k - 1), mom_mu(m, i, j - 1, k - 1)};
+    mom_cell<CONV, VISC, POW2>(m, n, c, i, j, k, mu);
+}
+
 // blocks as k_phi_grad's (W x R threads, at most kPhiThreads, RUN planes up z); the viscosities of a plane
 // of the block, with those of the row and the column before it, in one of three buffers by plane
 // (a buffer is written again three planes later: one barrier per plane)
-template <bool CONV, bool VISC, bool POW2, int RUN>
+template <bool CONV, bool POW2, int RUN>
 __global__ void k_mom_parts(MomArgs m)
 {
-    __shared__ double sh[VISC ? 3 : 1][VISC ? kPhiThreads + kPhiW + 4 : 1];  // (R + 1) (W + 1): at most 3 x 257
+    __shared__ double sh[3][kPhiThreads + kPhiW + 4];  // (R + 1) (W + 1): at most 3 x 257
     const int W = blockDim.x, R = blockDim.y, tx = threadIdx.x, ty = threadIdx.y;
     const int i = blockIdx.x * W + tx, j = blockIdx.y * R + ty;
     const bool in = i < m.nx && j < m.ny;
@@ -2547,31 +2582,15 @@ __global__ void k_mom_parts(MomArgs m)
             if (ty == 0) buf[0] = i > 0 || j > 0 ? mom_mu(m, i - 1, j - 1, k) : mc;
         }
     };
-    if (VISC) plane(k0 - 1, sh[(k0 + 2) % 3]);
+    plane(k0 - 1, sh[(k0 + 2) % 3]);
     for (int k = k0; k < k1; k++) {
-        double mc = 0, mx = 0, my = 0, mz = 0, mxy = 0, mxz = 0, myz = 0;
-        if (VISC) {
-            double *const b = sh[k % 3], *const bl = sh[(k + 2) % 3];
-            plane(k, b);
-            __syncthreads();
-            mc = b[at];
-            mx = b[at - 1];
-            my = b[at - P];
-            mxy = b[at - P - 1];
-            mz = bl[at];
-            mxz = bl[at - 1];
-            myz = bl[at - P];
-        }
+        double *const b = sh[k % 3], *const bl = sh[(k + 2) % 3];
+        plane(k, b);
+        __syncthreads();
+        const MomMu mu{b[at], b[at - 1], b[at - P], bl[at], b[at - P - 1], bl[at - 1], bl[at - P]};
         const size_t c = ((size_t)k * m.ny + j) * m.nx + i;
         if (!in || !MG_CK(c, c, (long long)n, CK_MOMENTUM)) continue;
-        mom_centre<0, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
-        mom_centre<1, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
-        mom_centre<2, CONV, VISC, POW2>(m, n, c, i, j, k, mc);
-        // in cell-index order: the cell below along both axes, below along the higher axis, below along
-        // the lower axis, the cell itself
-        mom_edge<0, 1, CONV, VISC, POW2>(m, n, c, i, j, k, mc, mx, my, mxy);
-        mom_edge<0, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mc, mx, mz, mxz);
-        mom_edge<1, 2, CONV, VISC, POW2>(m, n, c, i, j, k, mc, my, mz, myz);
+        mom_cell<CONV, true, POW2>(m, n, c, i, j, k, mu);
     }
 }
 
@@ -4118,28 +4137,30 @@ cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_a
     m.r = r;
     m.w = work;
     const dim3 g2 = row_grid2(d.nx, d.ny, d.nz), blk = row_block2(d.nx);
-    // Blocks of kPhiRun planes; on a grid that makes fewer than one block per SM so, of two planes and fewer rows:
-    // both passes 32^3 29 us (72 in blocks of eight planes), 48^3 39 (92), 64^3 66 (90).  At 96^3 (240 blocks) the longer
-    // runs are the faster ones, 223 us against 238: an edge is formed again at each end of a run.
+    // Where the viscosities are shared (k_mom_parts): not below 70,000 cells and not where a row fills less than 60 % of its
+    // blocks' lanes; in runs of two planes by 128 threads (or a row) below 3 M cells, of kPhiRun by kPhiThreads above.  Both
+    // passes with all terms, h a power of two; per cell, 2 and 8 planes, us: 16^3 10, 15, 65; 32^3 13, 16, 68; 48^3 33, 32, 76; 64^3 56, 51,
+    // 86; 80^3 121, 117, 157; 96^3 169, 163, 180; 128^3 390, 364, 390; 192x160x224 1260, 1177, 1212; 256^3 3040, 2854, 2767; narrow rows:
+    // 16x16x1024 56, 76, 84; 300x48x49 149, 157, 178; 2x600x600 144, 1087, 1101.  Without the viscous term per cell throughout:
+    // 64^3 25, 25, 36; 256^3 1269, 1270, 1289.
+    const bool two = d.n() < 3000000;
     dim3 pg, pb;
-    row_share_grid(d, pg, pb);
-    const bool few = (size_t)pg.x * pg.y * pg.z < 152;
-    for (int threads = kPhiThreads; few && threads >= 128; threads /= 2) {
-        row_share_grid(d, pg, pb, kMomRun, threads);
-        if ((size_t)pg.x * pg.y * pg.z >= 2 * 152) break;
-    }
+    row_share_grid(d, pg, pb, two ? kMomRun : kPhiRun, two ? 128 : kPhiThreads);
+    const bool share = d.n() >= 70000 && 5 * (size_t)d.nx >= 3 * (size_t)pg.x * pb.x;
     auto go = [&](auto conv, auto visc, auto pow2) {
         constexpr bool C = decltype(conv)::value, V = decltype(visc)::value, P = decltype(pow2)::value;
-        if (C || V) {
+        if constexpr (C || V) {
             note_launch();
-            if (few) k_mom_parts<C, V, P, kMomRun><<<pg, pb, 0, s>>>(m);
-            else k_mom_parts<C, V, P, kPhiRun><<<pg, pb, 0, s>>>(m);
+            if (!V || !share) k_mom_parts_cells<C, V, P><<<g2, blk, 0, s>>>(m);
+            else if (two) k_mom_parts<C, P, kMomRun><<<pg, pb, 0, s>>>(m);
+            else k_mom_parts<C, P, kPhiRun><<<pg, pb, 0, s>>>(m);
         }
         note_launch();
         k_mom_combine<C, V, P><<<g2, blk, 0, s>>>(m);
     };
     auto go_p = [&](auto conv, auto visc) {
-        if (m.ih.ok) go(conv, visc, BoolTag<true>{});
+        // (few cells wait for their chain of operations, on which the exponent shift is the longer one: 16^3 10.2 us, 9.4)
+        if (m.ih.ok && d.n() >= 30000) go(conv, visc, BoolTag<true>{});
         else go(conv, visc, BoolTag<false>{});
     };
     const BoolTag<true> yes;

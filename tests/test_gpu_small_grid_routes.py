@@ -63,3 +63,20 @@ def test_divergence_bit_exact_on_every_route(mgp, shape, areas, body):
         ctx.set_body_velocity(faces_dev(v))
     for dt in (1.0, 0.3):
         assert np.array_equal(host(ctx.divergence(faces_dev(u), dt=dt)), O.divergence_area(area, u, 1.0, dt, v))
+
+
+@pytest.mark.parametrize("inv_re,convection", [(0.37, True), (0.37, False), (0.0, True)])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (32, 33, 64), (64, 32, 35), (19, 61, 64), (20, 61, 64), (2, 190, 191),
+                                   (300, 20, 13), (308, 20, 13), (96, 31, 25), (144, 144, 145), (145, 144, 144),
+                                   (140, 150, 144)])
+def test_momentum_bit_exact_on_every_route(mgp, shape, inv_re, convection):
+    case = synth.small_case(*shape, seed=87, solid="none", interface="random", fields=False)
+    rng = np.random.default_rng(88)
+    u = [rng.standard_normal(case.shape) for _ in range(3)]
+    beta = O.face_coeffs(case.phi, None, case.lam)
+    for h in (case.h, 0.25):
+        want = O.momentum_rhs(case.phi, beta, u, h, g=1.3, inv_re=inv_re, mu_air=1.8e-2, convect=convection)
+        f = mgp.forces(g=1.3, inv_re=inv_re, mu_air=1.8e-2, convection=convection)
+        got = mgp.momentum_rhs(dev(case.phi), faces_dev(beta), faces_dev(u), h, f)
+        for a, b in zip(faces_host(got), want):
+            assert np.array_equal(a, b)
