@@ -3482,11 +3482,13 @@ inline dim3 row_grid2(int threads_x, int ny, int nz)
     return dim3((unsigned)((threads_x + b.x - 1) / b.x), (unsigned)((ny + b.y - 1) / b.y), (unsigned)nz);
 }
 
-// Blocks of the kernels that share values along rows: W x R threads, a row rounded up to whole warps (at
-// most kPhiW cells) by as many rows as fit, and `run` planes
+// Blocks of the kernels that share values along rows: W x R threads, a row or, beyond kPhiW cells, an equal part of
+// one, rounded up to whole warps, by as many rows as fit, and `run` planes.  (In parts of kPhiW a row of 300 cells left 41 % of
+// the lanes idle: face coefficients of 300x48x49 105 us, 67 so.)
 inline void row_share_grid(Dims d, dim3 &grid, dim3 &block, int run = kPhiRun, int threads = kPhiThreads)
 {
-    const int W = std::min((d.nx + 31) / 32 * 32, kPhiW), R = std::max(1, std::min(threads / W, d.ny));
+    const int parts = (d.nx + kPhiW - 1) / kPhiW, W = ((d.nx + parts - 1) / parts + 31) / 32 * 32;
+    const int R = std::max(1, std::min(threads / W, d.ny));
     grid = dim3((unsigned)((d.nx + W - 1) / W), (unsigned)((d.ny + R - 1) / R), (unsigned)((d.nz + run - 1) / run));
     block = dim3((unsigned)W, (unsigned)R);
 }
@@ -4137,16 +4139,16 @@ cudaError_t launch_momentum_rhs(Dims d, double h, const double *phi, double mu_a
     m.r = r;
     m.w = work;
     const dim3 g2 = row_grid2(d.nx, d.ny, d.nz), blk = row_block2(d.nx);
-    // Where the viscosities are shared (k_mom_parts): not below 70,000 cells and not where a row fills less than 60 % of its
-    // blocks' lanes; in runs of two planes by 128 threads (or a row) below 3 M cells, of kPhiRun by kPhiThreads above.  Both
+    // Where the viscosities are shared (k_mom_parts): not below 70,000 cells and not in rows of less than 20 cells, which
+    // leave a warp's lanes idle; in runs of two planes by 128 threads (or a row) below 3 M cells, of kPhiRun by kPhiThreads above.  Both
     // passes with all terms, h a power of two; per cell, 2 and 8 planes, us: 16^3 10, 15, 65; 32^3 13, 16, 68; 48^3 33, 32, 76; 64^3 56, 51,
     // 86; 80^3 121, 117, 157; 96^3 169, 163, 180; 128^3 390, 364, 390; 192x160x224 1260, 1177, 1212; 256^3 3040, 2854, 2767; narrow rows:
-    // 16x16x1024 56, 76, 84; 300x48x49 149, 157, 178; 2x600x600 144, 1087, 1101.  Without the viscous term per cell throughout:
+    // 16x16x1024 56, 76, 84; 2x600x600 144, 1087, 1101; 33x65x129 104, 97, 106; 33x300x300 1060 and, in 8 planes, 993.  Without the viscous term per cell throughout:
     // 64^3 25, 25, 36; 256^3 1269, 1270, 1289.
     const bool two = d.n() < 3000000;
     dim3 pg, pb;
     row_share_grid(d, pg, pb, two ? kMomRun : kPhiRun, two ? 128 : kPhiThreads);
-    const bool share = d.n() >= 70000 && 5 * (size_t)d.nx >= 3 * (size_t)pg.x * pb.x;
+    const bool share = d.n() >= 70000 && d.nx >= 20;
     auto go = [&](auto conv, auto visc, auto pow2) {
         constexpr bool C = decltype(conv)::value, V = decltype(visc)::value, P = decltype(pow2)::value;
         if constexpr (C || V) {

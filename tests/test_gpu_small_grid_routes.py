@@ -80,3 +80,24 @@ def test_momentum_bit_exact_on_every_route(mgp, shape, inv_re, convection):
         got = mgp.momentum_rhs(dev(case.phi), faces_dev(beta), faces_dev(u), h, f)
         for a, b in zip(faces_host(got), want):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(257, 9, 11), (300, 48, 49), (449, 5, 17), (512, 3, 9), (513, 7, 10), (705, 4, 8)])
+def test_rows_of_several_blocks_bit_exact(mgp, shape):
+    """Rows longer than a block are cut into equal parts of whole warps: face coefficients, their adjoint, and
+    the momentum terms over the cuts."""
+    case = synth.small_case(*shape, seed=89, solid="ellipsoid", interface="random", fields=False)
+    rng = np.random.default_rng(90)
+    field = lambda: [rng.standard_normal(case.shape) for _ in range(3)]
+    for solid in (None, case.solid):
+        beta = O.face_coeffs(case.phi, solid, case.lam)
+        got = mgp.face_coeffs(dev(case.phi), case.h, None if solid is None else dev(solid, torch.uint8), rho_air=case.lam)
+        for a, b in zip(faces_host(got), beta):
+            assert np.array_equal(a, b)
+        gb, u = field(), field()
+        g = mgp.phi_grad(faces_dev(beta), faces_dev(gb), case.h, rho_air=case.lam)
+        assert np.array_equal(host(g), O.phi_grad(beta, gb, case.lam))
+        want = O.momentum_rhs(case.phi, beta, u, case.h, g=1.3, inv_re=0.37, mu_air=1.8e-2, convect=True)
+        f = mgp.forces(g=1.3, inv_re=0.37, mu_air=1.8e-2, convection=True)
+        for a, b in zip(faces_host(mgp.momentum_rhs(dev(case.phi), faces_dev(beta), faces_dev(u), case.h, f)), want):
+            assert np.array_equal(a, b)
