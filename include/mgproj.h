@@ -105,7 +105,7 @@ typedef struct {
                              finest) as one CUDA graph captured on first use on a private stream;
                              0: launch its kernels one by one.  Identical results [1] */
     int coarse_tail;      /* 1: the levels of at most 8192 cells below the finest, the coarsest solve
-                             included (up to 1024 cells), run in one launch of one thread-block
+                             included (up to 512 cells), run in one launch of one thread-block
                              cluster instead of a launch per pass; 0: a launch per pass.  Identical
                              results [1] */
     int precond;          /* preconditioner of the conjugate gradients (krylov = 1): 0 inner_cycles

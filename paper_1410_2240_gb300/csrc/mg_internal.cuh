@@ -120,7 +120,11 @@ constexpr int kTailThreads = 256, kTailCells = 2;  // per CTA, and cells of a co
 // FP64 unit of 16 SMs).
 constexpr size_t kTailCellsMax = 8192;
 constexpr size_t kTailSmem = 128 * 1024;   // shared memory per CTA at most (8192 FP64 cells need half)
-constexpr int kTailCoarse = 1024;          // cells of the coarsest grid at most
+// Cells of the coarsest grid at most: its inverse is read by the cluster's 16 SMs, by a launch of its own on all of them.
+// V-cycle of a grid two levels above it with 2 + 2 and 1 + 1 sweeps, in the tail and by launches, us: FP64 256 cells 62 and 72, 44 and
+// 48; 448 cells 68 and 70, 50 and 50; 504 cells 74 and 74, 54 and 50; 660 cells 75 and 72, 56 and 50; 840 cells 81 and 75, 62 and 50;
+// 990 cells 91 and 76, 70 and 52.  FP32 256 cells 66 and 72, 49 and 53; 504 cells 77 and 75, 61 and 55; 840 cells 88 and 77, 69 and 57.
+constexpr int kTailCoarse = 512;
 template <typename T>
 struct TailLevel {
     int nx, ny, nz;

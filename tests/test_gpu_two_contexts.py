@@ -13,8 +13,9 @@ from _gpu_util import dev, host
 
 pytestmark = pytest.mark.gpu
 
-# tails that start at 32x32x8, 8x8x8 and 16^3: 71, 4 and 20 KB of shared memory per CTA in FP64
-SHAPES = [(64, 64, 16), (16, 16, 16), (32, 32, 32)]
+# tails that start at 20^3, 8^3 and 16^3: 50, 4 and 20 KB of shared memory per CTA in FP64 (48 KB is what a kernel
+# has without asking)
+SHAPES = [(40, 40, 40), (16, 16, 16), (32, 32, 32)]
 
 
 @pytest.fixture(scope="module")
@@ -105,3 +106,18 @@ def test_contexts_in_two_threads(mgp, prec, graph):
     for th in threads:
         th.join()
     assert not failed, failed
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape,tail", [((32, 64, 32), True), ((28, 32, 36), True), ((36, 36, 28), False), ((36, 36, 36), False)])
+def test_tail_up_to_512_cells_of_the_coarsest_grid(mgp, shape, tail, prec):
+    """Coarsest grids of 256, 504, 567 and 729 cells: a larger one is solved by a launch of its own on every SM."""
+    launches = []
+    for t in (0, 1):
+        ctx, rhs = _make(mgp, shape, prec=prec, coarse_tail=t)
+        p = torch.zeros_like(rhs)
+        l0 = mgp.kernel_launches()
+        ctx.vcycle(rhs, p)
+        launches.append(mgp.kernel_launches() - l0)
+        ctx.close()
+    assert (launches[1] < launches[0]) == tail
