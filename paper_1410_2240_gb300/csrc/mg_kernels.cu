@@ -588,6 +588,15 @@ GsScale<T> gs_scale(T h2)
 // addition, those of a product's factors are free.
 __device__ __forceinline__ double gs_start(double b, const GsScale<double> &g) { return mul_s2(b, g.s); }
 __device__ __forceinline__ float gs_start(float, const GsScale<float> &) { return 0.f; }
+// the same with the kind of the factor known to the kernel (POW2; FP32: not asked): a product that is none of the shift's
+// is a multiplication in place, where gs_start makes a call
+template <bool POW2>
+__device__ __forceinline__ double gs_start_of(double b, const GsScale<double> &g)
+{
+    return POW2 ? mul_pow2(b, g.s.f, g.s.e) : __dmul_rn(b, g.s.f);
+}
+template <bool POW2>
+__device__ __forceinline__ float gs_start_of(float, const GsScale<float> &) { return 0.f; }
 __device__ __forceinline__ double gs_add(double beta, double p, double s) { return fma(beta, -p, s); }
 __device__ __forceinline__ float gs_add(float beta, float p, float s) { return fmaf(beta, p, s); }
 __device__ __forceinline__ double gs_update(double s, double, double d, const GsScale<double> &) { return -d * s; }
@@ -1649,7 +1658,7 @@ __global__ void k_prolong_black(int nx, int ny, int nz, float h2, LevelArrays<fl
 // Shared memory holds three rotating planes of (p, bx, by): the x+ and y+ face
 // coefficients of a cell are its neighbour's low faces.
 // ---------------------------------------------------------------------------
-template <typename T, int TX, int TY>
+template <typename T, bool POW2, int TX, int TY>
 __global__ void __launch_bounds__((TX + 4) * (TY + 4))
 k_rb_sweep(int nx, int ny, int nz, int zc, GsScale<T> gs, LevelArrays<T> L, const T *__restrict__ b,
            const T *__restrict__ p_old, T *__restrict__ p_new, int first)
@@ -1706,7 +1715,7 @@ k_rb_sweep(int nx, int ny, int nz, int zc, GsScale<T> gs, LevelArrays<T> L, cons
         if (ring1 && s >= 0 && s < nz && ((i + j + s) & 1) == first) {
             const T bxh = xhi ? sbx[cur][ly][lx + 1] : T(0), byh = yhi ? sby[cur][ly + 1][lx] : T(0);
             const T bzh = (s < nz - 1) ? bz_p1 : T(0);
-            T acc = gs_start(b_0, gs);
+            T acc = gs_start_of<POW2>(b_0, gs);
             if (xlo) acc = gs_add(bx_0, sp[cur][ly][lx - 1], acc);
             if (xhi) acc = gs_add(bxh, sp[cur][ly][lx + 1], acc);
             if (ylo) acc = gs_add(by_0, sp[cur][ly - 1][lx], acc);
@@ -1723,7 +1732,7 @@ k_rb_sweep(int nx, int ny, int nz, int zc, GsScale<T> gs, LevelArrays<T> L, cons
             if (((i + j + z) & 1) == second) {
                 const T bxh = xhi ? sbx[prv][ly][lx + 1] : T(0), byh = yhi ? sby[prv][ly + 1][lx] : T(0);
                 const T bzh = (z < nz - 1) ? bz_0 : T(0);
-                T acc = gs_start(b_m1, gs);
+                T acc = gs_start_of<POW2>(b_m1, gs);
                 if (xlo) acc = gs_add(bx_m1, sp[prv][ly][lx - 1], acc);
                 if (xhi) acc = gs_add(bxh, sp[prv][ly][lx + 1], acc);
                 if (ylo) acc = gs_add(by_m1, sp[prv][ly - 1][lx], acc);
@@ -3811,8 +3820,12 @@ cudaError_t launch_rb_sweep(Dims d, T h2, const LevelArrays<T> &L, const T *b, c
     if (zc > d.nz) zc = d.nz;
     const dim3 grid((unsigned)tx, (unsigned)ty, (unsigned)((d.nz + zc - 1) / zc));
     note_launch();
-    k_rb_sweep<T, TX, TY><<<grid, (TX + 4) * (TY + 4), 0, s>>>(d.nx, d.ny, d.nz, zc, gs_scale<T>(h2), L, b, p_old, p_new,
-                                                              first);
+    // (FP64, h no power of two: 256^3, V-cycle of 2 + 2 such sweeps: 4.09 ms, 4.47 with gs_start's call per cell)
+    const GsScale<T> gs = gs_scale<T>(h2);
+    if (sizeof(T) == 4 || gs.s.ok)
+        k_rb_sweep<T, true, TX, TY><<<grid, (TX + 4) * (TY + 4), 0, s>>>(d.nx, d.ny, d.nz, zc, gs, L, b, p_old, p_new, first);
+    else if constexpr (sizeof(T) == 8)
+        k_rb_sweep<T, false, TX, TY><<<grid, (TX + 4) * (TY + 4), 0, s>>>(d.nx, d.ny, d.nz, zc, gs, L, b, p_old, p_new, first);
     return cudaGetLastError();
 }
 template cudaError_t launch_rb_sweep<double>(Dims, double, const LevelArrays<double> &, const double *,

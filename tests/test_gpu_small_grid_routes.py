@@ -101,3 +101,20 @@ def test_rows_of_several_blocks_bit_exact(mgp, shape):
         f = mgp.forces(g=1.3, inv_re=0.37, mu_air=1.8e-2, convection=True)
         for a, b in zip(faces_host(mgp.momentum_rhs(dev(case.phi), faces_dev(beta), faces_dev(u), case.h, f)), want):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("h", [0.25, 0.3])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_fused_sweeps_with_any_spacing_identical_to_passes(mgp, prec, h):
+    """h^2 b is an exponent shift or a multiplication, chosen by h: the fused sweep's choice against the passes'."""
+    case = synth.small_case(72, 40, 48, seed=91, solid="ellipsoid", fields=False)
+    beta = mgp.face_coeffs(dev(case.phi), h, dev(case.solid, torch.uint8), rho_air=case.lam)
+    rhs = dev(np.random.default_rng(92).standard_normal(case.shape))
+    out = []
+    for sm in (1, 2):
+        ctx = mgp.Context(beta, h, prec=prec, smoother=sm, coarse_max_cells=2048)
+        p = torch.zeros_like(rhs)
+        for _ in range(2):
+            ctx.vcycle(rhs, p)
+        out.append(p)
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
