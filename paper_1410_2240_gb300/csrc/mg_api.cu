@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <initializer_list>
+#include <memory>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -341,10 +342,13 @@ int coarse_inverse(int nx, int ny, int nz, double h, const double *bx, const dou
         const int groups = (m + kInvCols - 1) / kInvCols;
         std::vector<double> r(m);
         double all = 0.0;
-        std::vector<double> work((size_t)(m > 128 ? omp_get_max_threads() : 1) * m * kInvCols);
-#pragma omp parallel if (m > 128)
+        // a part per thread, none of it read before it is written (clearing one per thread of a large host, most of them
+        // without a group of columns, took longer than the columns)
+        const int team = m > 128 ? std::min(omp_get_max_threads(), groups) : 1;
+        const std::unique_ptr<double[]> work(new double[(size_t)team * m * kInvCols]);
+#pragma omp parallel num_threads(team)
         {
-            double *const W = &work[(size_t)omp_get_thread_num() * m * kInvCols];  // rows j0 .. m - 1
+            double *const W = work.get() + (size_t)omp_get_thread_num() * m * kInvCols;  // rows j0 .. m - 1
 #pragma omp for schedule(dynamic, 1)
             for (int gr = 0; gr < groups; gr++) {
                 const int j0 = gr * kInvCols, nc = std::min(kInvCols, m - j0);
