@@ -105,7 +105,7 @@ def parse_args():
     ap.add_argument("--smoother", type=int, default=0,
                     help="0 auto, 1 per colour, 2 fused, 3 fused + TMA")
     ap.add_argument("--coarse-tail", type=int, default=1,
-                    help="smallest levels: 0 a launch per pass, 1 one CTA (coarse_tail option)")
+                    help="smallest levels: 0 a launch per pass, 1 one thread-block cluster (coarse_tail option)")
     ap.add_argument("--pass-order", type=int, default=1,
                     help="finest colour passes: 1 alternate descending/ascending plane order (L2 reuse), 0 ascending")
     ap.add_argument("--krylov", type=int, default=1,

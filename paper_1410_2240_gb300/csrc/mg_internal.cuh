@@ -162,7 +162,7 @@ cudaError_t launch_level_f32(Dims d, const LevelArrays<double> &L, LevelArrays<f
 
 // one colour of a red-black sweep; zero: the iterate is zero and is not read (the first pass of a
 // cycle from a zero guess)
-// rec (FP64, optional): the level's row records (launch_row_records64)
+// rec (optional): the level's row records (launch_row_records)
 template <typename T>
 cudaError_t launch_smooth(Dims d, T h2, const LevelArrays<T> &L, const T *b, T *p, int colour, cudaStream_t s,
                           bool zero = false, const T *rec = nullptr, Gate gate = {});

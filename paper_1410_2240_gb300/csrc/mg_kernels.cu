@@ -336,12 +336,12 @@ __device__ __forceinline__ double mul_pow2(double x, double f, int e)
 #endif
     return y;
 }
-// the product with a power-of-two factor (ok: f = 2^e) or any other (ok = 0: a multiply)
 // -x, exactly, on the integer pipe (a negation that no operand takes is an FP64 addition)
 __device__ __forceinline__ double neg_bits(double x)
 {
     return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
 }
+// the product with a power-of-two factor (ok: f = 2^e) or any other (ok = 0: a multiply)
 __device__ __forceinline__ double mul_s2(double x, const Scale2 &s) { return s.ok ? mul_pow2(x, s.f, s.e) : dmul_call(x, s.f); }
 
 // cell c = (i, j, k) and the neighbours its guards admit (i > 0: c - 1, i < nx - 1: c + 1, ...)
@@ -610,7 +610,8 @@ __device__ __forceinline__ float gs_update(float s, float b, float d, const GsSc
 // much as by the FP64 unit (0.132 ms at 8 operations, 0.115 at 7).  Sweep at 256^3, FP64: 0.271 ms with
 // 8 operations and every face loaded, 0.257 with 7 and the short zero pass, 0.231 with the records
 // too (the average over the passes of a cycle from zero); 128^3 40.6 -> 34.2 us.
-// FP32, a coarse level of 512 x 256 x 128: 54.6 us per pass.
+// Where h is no power of two an update is 8 operations, the eighth in a call: V-cycle at 256^3 1.55 ms, 1.67 with h = 1/30 (2.09 with
+// both before).  FP32 coarse levels: kRecCells32 has both sides.
 // GATE: a pass queued before the host knows whether the iteration has ended: it stores nothing unless the squared
 // residual norm *gate.rr is finite and above gate.limit (both compared as integers: not negative).
 template <typename T, bool ZERO, bool ROWS, bool GATE = false>
@@ -1027,27 +1028,12 @@ __global__ void k_smooth_split4(int nx, int ny, int nz, float h2, LevelArrays<fl
     else split4_body<1, 0, BAND, ZERO>(nx, ny, nz, h2, S, b, p, colour, rv, iv, g, j, k, 0, dinv);
 }
 
-// r = b - h^-2 sum_f beta_f (p_nb - p_c) at one fine cell (sum order x-,x+,y-,y+,z-,z+).
-template <typename T>
-__device__ __forceinline__ T residual_at(int i, int j, int k, size_t c, int nx, int ny, int nz, size_t sxy, T ih2,
-                                         const LevelArrays<T> &L, const T *b, const T *p)
-{
-    if (!ck_cell((long long)c, i, j, k, nx, ny, nz, CK_RESID)) return T(0);
-    const T pc = p[c];
-    T s = T(0);
-    if (i > 0) s = fma(L.bx[c], p[c - 1] - pc, s);
-    if (i < nx - 1) s = fma(L.bx[c + 1], p[c + 1] - pc, s);
-    if (j > 0) s = fma(L.by[c], p[c - nx] - pc, s);
-    if (j < ny - 1) s = fma(L.by[c + nx], p[c + nx] - pc, s);
-    if (k > 0) s = fma(L.bz[c], p[c - sxy] - pc, s);
-    if (k < nz - 1) s = fma(L.bz[c + sxy], p[c + sxy] - pc, s);
-    return fma(-s, ih2, b[c]);
-}
-
 // FP64 residuals for the solver's convergence checks: f(c, (j + k) & 1, r, p_c) for every cell.  The blocks
 // take tasks of 256 columns by `run` planes; a thread walks up its column and takes the difference to the cell
 // below from the step before (its negative, exactly): 12 FP64 operations for a residual instead of 13, two
-// loads less (with the norm, 59 us at 128^3, 68 us with one thread per cell and the sum of p in the same pass).  The terms and their order are residual_at's.  Where p and its in-domain neighbours are
+// loads less (with the norm, 59 us at 128^3, 68 us with one thread per cell and the sum of p in the same pass).
+// r = b - h^-2 sum_f beta_f (p_nb - p_c), summed x-, x+, y-, y+, z-, z+: differences of neighbouring p first, so a
+// large smooth offset in p (a hydrostatic pressure) cancels before any product.  Where p and its in-domain neighbours are
 // all zero (bitwise, either sign) every product beta (0 - 0) is a signed zero, the sum stays +0
 // and the residual is b[c] exactly (for finite coefficients): the test runs on the integer
 // pipe and skips the FP64 arithmetic, which dominates this pass on a zero initial guess.
@@ -2025,7 +2011,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
 // ---------------------------------------------------------------------------
 // The passes below read one or two arrays once.  Each thread takes two pairs of cells per iteration, all
 // loads issued first: at one cell per iteration their five blocks per SM left HBM at half its rate.
-// f(pair index, true) for two pairs at a time is loads(v) -> use(v, ...); the last cell of an odd n is cell(n - 1).
+// load(v) returns what pair v (cells 2v and 2v + 1) needs, use(v, that) works on it; the last cell of an odd n is cell(n - 1).
 template <typename Load, typename Use, typename Cell>
 __device__ __forceinline__ void stream_pairs(unsigned n, Load load, Use use, Cell cell)
 {
@@ -2965,9 +2951,7 @@ __global__ void k_nonzero(unsigned n, const double *__restrict__ p, unsigned *__
     if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(flag, 1u);
 }
 
-// r = b - A p (FP64), as residual_at forms it: differences of neighbouring p first, so a large
-// smooth offset in p (a hydrostatic pressure) cancels before any product.  Optionally r32 = r /
-// scale, scale = RMS of b (first pass) written to scale_slot.
+// r = b - A p (FP64, resid_columns).  Optionally r32 = r / scale, scale = RMS of b (first pass) written to scale_slot.
 // pnz (optional): the k_nonzero flag of p; 0 means p is zero everywhere, and each cell's
 // residual is then b exactly with no stencil loaded: the same values for a fraction of the loads (the
 // first residual of a solve from a zero guess), streamed as pairs of cells in a loop that holds no stencil
