@@ -827,7 +827,7 @@ int final_status(mg_ctx *c, int status)
 }
 
 // p -= its mean over each fluid region (live cells), dead cells 0; with one region the mean is
-// dscal[S_SUM_P] / nlive, from the CG's last residual pass or (sum) summed here
+// dscal[S_SUM_P] / nlive, from the last residual pass or (sum) summed here
 int remove_p_mean(mg_ctx *c, double *p, bool sum)
 {
     const Dims d = c->dims[0];
@@ -844,7 +844,9 @@ int remove_p_mean(mg_ctx *c, double *p, bool sum)
 // Colour passes of the next cycle to queue before the host waits for a residual: the GPU would stand idle for the
 // copy, the host's wait and the next launch, some 13 us an iteration (a tenth of one at 64^3).  As many as take some
 // 20 us (a pass moves about three values per cell at 4 TB/s), at least one; none where the cycle is not
-// made of colour passes or is timed by parts.
+// made of colour passes or is timed by parts.  Anything from 10 to 40 us gives the same: mixed CG solves of 32^3, 64^3, 96^3 and 128^3
+// with none ahead 1176, 1820, 2280 and 3074 us, with 5 us of passes 1152, 1805, 2259, 3027, 10 us 1140, 1777, 2251, 3025, 20 us 1145,
+// 1782, 2260, 3023, 40 us 1145, 1777, 2266, 3056.
 int passes_ahead(const mg_ctx *c)
 {
     const bool mixed = c->o.prec == MG_MIXED;
@@ -939,7 +941,7 @@ int solve_impl(mg_ctx *c, const double *rhs, double *p, double tol, mg_stats *st
     }
     // zero mean over each region's live cells (the cycle commutes with constant shifts, so once
     // suffices)
-    CKS(remove_p_mean(c, p, true));
+    CKS(remove_p_mean(c, p, !mg::resid_sums_p(d.n())));
     CK(cudaEventRecord(c->ev1, s));
     CK(cudaEventSynchronize(c->ev1));
     if (st) {

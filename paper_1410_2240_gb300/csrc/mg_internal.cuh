@@ -260,6 +260,11 @@ cudaError_t launch_rhs_prepare(Dims d, const double *rhs, const double *dinv, do
                                double *dscal, cudaStream_t s);
 cudaError_t launch_resid_norm(Dims d, double ih2, const LevelArrays<double> &L, const double *b, const double *p,
                               double *partials, double *dscal, cudaStream_t s);
+// Whether launch_resid_norm and launch_resid_cast write dscal[S_SUM_P] too, so that the mean of p a solve removes at its end
+// takes no pass of its own (launch_sum_p): on small grids, where a pass is a launch.  Solves with a pass of its own and without, us: 5x7x9
+// 91 and 87, 16^3 780 and 755, 32^3 1116 and 1114, 64^3 2028 and 2025; 96^3 3503 and 3542, 128^3 5950 and 6039, mixed 3771 and 3943 (the
+// sum's FP64 additions in every residual).
+inline bool resid_sums_p(size_t n) { return n <= 65536; }
 // dscal[S_SUM_P] = the sum of p over the live cells (launch_pcg_resid writes it too)
 cudaError_t launch_sum_p(Dims d, const double *dinv, const double *p, double *partials, double *dscal, cudaStream_t s);
 cudaError_t launch_sub_mean_p(Dims d, const double *dinv, double *p, const double *dscal, cudaStream_t s);

@@ -2079,14 +2079,19 @@ __global__ void k_rhs_center(unsigned n, const double *__restrict__ rhs, const d
     reduce_finish(block_sum<kRedThreads>(a), 0.0, partials, dscal, S_NB2, -1);
 }
 
-// ||b - A p||^2
+// ||b - A p||^2; SUM: and the sum of p over the live cells (resid_sums_p)
+template <bool SUM>
 __global__ void k_resid_norm(int nx, int ny, int nz, double ih2, LevelArrays<double> L,
                              const double *__restrict__ b, const double *__restrict__ p, double *__restrict__ partials,
                              double *dscal, ResidGrid g)
 {
-    double rr = 0.0;
-    resid_columns(nx, ny, nz, ih2, L, b, p, g, [&](size_t, int, double r, double) { rr = fma(r, r, rr); });
-    reduce_finish(block_sum<kRedThreads>(rr), 0.0, partials, dscal, S_RR, -1);
+    double rr = 0.0, sum = 0.0;
+    resid_columns(nx, ny, nz, ih2, L, b, p, g, [&](size_t c, int, double r, double pc) {
+        rr = fma(r, r, rr);
+        if (SUM && pos_bits(L.dinv[c])) sum += pc;
+    });
+    block_sum2<kRedThreads, SUM>(rr, sum);
+    reduce_finish(rr, sum, partials, dscal, S_RR, SUM ? S_SUM_P : -1);
 }
 
 // p -= mean of p over live cells (mean = dscal[S_SUM_P] / dscal[S_NLIVE]); dead cells 0
@@ -2104,21 +2109,23 @@ __global__ void k_sub_mean_p(unsigned n, const double *__restrict__ dinv, double
 }
 
 // Mixed refinement: r = b - A p in FP64, stored as FP32 r / scale_in; partial ||r||^2.
+template <bool SUM>
 __global__ void k_resid_cast(int nx, int ny, int nz, double ih2, LevelArrays<double> L,
                              const double *__restrict__ b, const double *__restrict__ p, float *__restrict__ r32,
                              double *dscal, int scale_in, int scale_out, double *__restrict__ partials, size_t half,
                              ResidGrid g)
 {
     const double inv_scale = block_scalar([&] { return 1.0 / dscal[scale_in]; });
-    double rr = 0.0;
-    resid_columns(nx, ny, nz, ih2, L, b, p, g, [&](size_t c, int q, double r, double) {
+    double rr = 0.0, sum = 0.0;
+    resid_columns(nx, ny, nz, ih2, L, b, p, g, [&](size_t c, int q, double r, double pc) {
         rr = fma(r, r, rr);
+        if (SUM && pos_bits(L.dinv[c])) sum += pc;
         const size_t slot = half ? split_slot(c, q, half) : c;
         if (MG_CK(slot, slot, (long long)nx * ny * nz, CK_SPLIT_SLOT)) r32[slot] = narrow(r * inv_scale);
     });
-    rr = block_sum<kRedThreads>(rr);
+    block_sum2<kRedThreads, SUM>(rr, sum);
     // the last block also sets the next scale: the RMS of this residual over the live cells (1 if 0)
-    if (reduce_finish(rr, 0.0, partials, dscal, S_RR, -1) && threadIdx.x == 0 && scale_out >= 0) {
+    if (reduce_finish(rr, sum, partials, dscal, S_RR, SUM ? S_SUM_P : -1) && threadIdx.x == 0 && scale_out >= 0) {
         const double rms = sqrt(dscal[S_RR] / dscal[S_NLIVE]);
         dscal[scale_out] = (rms > 0.0 && isfinite(rms)) ? rms : 1.0;
     }
@@ -3995,7 +4002,10 @@ cudaError_t launch_resid_norm(Dims d, double ih2, const LevelArrays<double> &L, 
 {
     const ResidGrid g = resid_grid(d);
     note_launch();
-    k_resid_norm<<<resid_blocks(g), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, ih2, L, b, p, partials, dscal, g);
+    if (resid_sums_p(d.n()))
+        k_resid_norm<true><<<resid_blocks(g), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, ih2, L, b, p, partials, dscal, g);
+    else
+        k_resid_norm<false><<<resid_blocks(g), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, ih2, L, b, p, partials, dscal, g);
     return cudaGetLastError();
 }
 
@@ -4024,8 +4034,12 @@ cudaError_t launch_resid_cast(Dims d, double ih2, const LevelArrays<double> &L, 
         k_scale_from_nb2<<<1, 1, 0, s>>>(dscal, scale_in);
     }
     note_launch();
-    k_resid_cast<<<resid_blocks(g), kRedThreads, 0, s>>>(d.nx, d.ny, d.nz, ih2, L, b, p, r32, dscal, scale_in, scale_out,
-                                                          partials, sp.half, g);
+    auto go = [&](auto sum) {
+        k_resid_cast<decltype(sum)::value><<<resid_blocks(g), kRedThreads, 0, s>>>(
+            d.nx, d.ny, d.nz, ih2, L, b, p, r32, dscal, scale_in, scale_out, partials, sp.half, g);
+    };
+    if (resid_sums_p(d.n())) go(BoolTag<true>{});
+    else go(BoolTag<false>{});
     return cudaGetLastError();
 }
 

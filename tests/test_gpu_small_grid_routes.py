@@ -118,3 +118,20 @@ def test_fused_sweeps_with_any_spacing_identical_to_passes(mgp, prec, h):
             ctx.vcycle(rhs, p)
         out.append(p)
     assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape", [(5, 7, 9), (64, 32, 32), (64, 32, 40)])
+def test_mean_of_p_removed_on_either_route(mgp, shape, prec):
+    """A solve of no cycle returns its guess without its mean over the live cells, summed in the residual's pass or in one
+    of its own: the sum of n terms is off by at most n 2^-53 of the largest of them."""
+    case = synth.small_case(*shape, seed=93, solid="none" if shape[0] == 5 else "ellipsoid", fields=False)
+    solid = case.solid
+    beta = O.face_coeffs(case.phi, solid, case.lam)
+    live = np.ones(case.shape, bool) if solid is None else solid == 0
+    p = np.random.default_rng(94).standard_normal(case.shape) + 3.0
+    ctx = mgp.Context(faces_dev(beta), case.h, prec=prec, max_cycles=0, coarse_max_cells=2048)
+    rhs = np.where(live, np.random.default_rng(95).standard_normal(case.shape), 0.0)
+    got, _ = ctx.solve(dev(rhs), dev(p), tol=1e-300, allow_not_converged=True)
+    want = np.where(live, p - p[live].mean(), 0.0)
+    assert np.abs(host(got) - want).max() <= p.size * 2.0 ** -53 * np.abs(p).max() + 1e-13
