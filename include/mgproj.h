@@ -421,7 +421,8 @@ int mg_level_array(mg_ctx *c, int level, int which, double *out);
  * time (ms, CUDA events on the context's stream) of one kernel group since the
  * last mg_profile_reset; the stream must be idle (any solve returns so).
  * Groups: 0 = one finest-grid red-black smoothing sweep (both colours, in the
- * precision the cycles run in), 1 = finest-grid residual + restriction, 2 =
+ * precision the cycles run in; the black pass that a cycle continuing another
+ * starts with is not timed), 1 = finest-grid residual + restriction, 2 =
  * finest-grid prolongation, 3 = FP64 finest-grid residual (norm, mixed cast,
  * or the conjugate-gradient update), 4 = conjugate-gradient operator apply
  * q = A d, 5 = conjugate-gradient dot products and direction update, 6 = all

@@ -636,7 +636,7 @@ int vcycle(mg_ctx *c, const std::vector<LevelArrays<T>> &L, int l, const T *b, T
             CKS(sweep(0));
             continue;
         }
-        ProfScope ps(c, MG_PROF_SMOOTH, fine);
+        ProfScope ps(c, MG_PROF_SMOOTH, fine && !(skip && it == 0));  // (a lone black pass is no sweep)
         for (int colour = 0; colour < 2; colour++) {
             const int m = 2 * it + colour;
             if (both && m < 2) {

@@ -100,3 +100,21 @@ def test_tail_runs_and_is_the_launches(mgp, shape, prec):
             launches.append(mgp.kernel_launches() - l0)
         assert launches[1] < launches[0]
         assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (1, 1), (2, 0)])
+@pytest.mark.parametrize("prec,krylov,inner", [("fp64", 0, 1), ("mixed", 0, 2), ("fp64", 1, 2)])
+def test_profiled_sweeps_are_whole_sweeps(mgp, prec, krylov, inner, nu):
+    """Group 0 times sweeps of both colours: a cycle that continues another starts with a black pass alone
+    (where it smooths on both ways), which is not one of them."""
+    case = synth.small_case(48, 16, 24, solid="ellipsoid", seed=97)
+    beta = mgp.face_coeffs(dev(case.phi), case.h, dev(case.solid, dtype=torch.uint8), rho_air=case.lam)
+    rhs = mgp.Context(beta, case.h, coarse_max_cells=2048).divergence(tuple(dev(u) for u in case.u_star))
+    ctx = mgp.Context(beta, case.h, prec=prec, krylov=krylov, inner_cycles=inner, nu1=nu[0], nu2=nu[1], profile=1,
+                      max_cycles=3, coarse_max_cells=2048)
+    _, st = ctx.solve(rhs, tol=1e-30, allow_not_converged=True)
+    assert st.cycles == 3
+    sweeps, _ = ctx.profile_read(mgp.PROF_SMOOTH)
+    cycles = 3 * (inner if prec == "mixed" or krylov else 1)
+    continued = (2 if krylov == 0 and prec == "fp64" else 3 * (inner - 1)) if nu[1] else 0
+    assert sweeps == cycles * sum(nu) - continued
