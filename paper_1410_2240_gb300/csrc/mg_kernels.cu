@@ -887,9 +887,9 @@ __global__ void k_smooth_split(int nx, int ny, int nz, float h2, LevelArrays<flo
 // and mb + hxy; six float4 and one scalar, each value used.
 // A record's two inverse diagonals are read from uinv (k_uniform_rows), and only a row's first cell (OFF = 0) or its
 // last one (OFF = 1) can lie at an x-wall: without the two divisions and eight wall tests per thread a sweep
-// takes 53.5 us at 256^3 instead of 56.2, 192x160x224 26.3 (30.1), 320x192x128 33.1 (37.1), 128^3 14.4 (15.6).  The
-// pass waits for its loads (half of the issue slots are used): 72 % of the copy rate at 256^3.  More warps
-// in fewer registers (48, 40: spills) take 63.0 and 67.5 us.
+// takes 56.9 us at 256^3 instead of 59.4, 192x160x224 27.9 (31.6), 320x192x128 35.3 (39.5), 128^3 15.3 (16.7).  The
+// pass waits for its loads (half of the issue slots are used): 67 % of the copy rate at 256^3.  More warps
+// in fewer registers (48, 40: spills) take 12 and 20 % longer.
 // ROWS: 1 where a warp lies in one row (OFF_ is then the row's offset), 0 where it may hold several
 // rows of both parities (off: this thread's; selected per value, so that the warp does not run the
 // two parities one after the other).
@@ -3496,9 +3496,9 @@ inline void row_share_grid(Dims d, dim3 &grid, dim3 &block, int run = kPhiRun, i
 // Blocks of the finest FP32 level's kernels that take several cells along x per thread (rows of G threads):
 // 32 threads by 4 rows where G is a multiple of 32, else G cut into equal parts of at most 32 threads
 // by as many rows as make up to 128 threads, so that short rows do not leave lanes idle (at nx = 128 a
-// colour pass had 16 threads per row and ran half of each warp: 18.4 us per sweep, 15.6 us so; 192x160x224
-// 33.0 -> 30.4 us, 320x192x128 43.2 -> 37.2 us).  Rows of 32 threads keep the colour pass's body per row
-// parity: with the parity selected per value it took 63.5 us per sweep at 256^3 instead of 57.8.
+// colour pass had 16 threads per row and ran half of each warp: 19.5 us per sweep, 16.5 us so; 192x160x224
+// 34.9 -> 31.8 us, 320x192x128 44.9 -> 39.6 us).  Rows of 32 threads keep the colour pass's body per row
+// parity: with the parity selected per value a sweep took 10 % longer at 256^3.
 inline dim3 pair_block(int G)
 {
     const int parts = (G + 31) / 32, x = (G + parts - 1) / parts;
